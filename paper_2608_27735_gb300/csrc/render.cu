@@ -13,12 +13,12 @@
 // pixels have terminated.  List entries are staged in shared memory; an entry whose opacity
 // cannot reach alpha_min anywhere on the CTA's pixel-centre box (analytic minimum of the
 // quadratic form over the box, with a margin far above fp32 rounding) is dropped while
-// staging -- every pixel would skip it, so results are unchanged -- and staging keeps loading
-// groups of 64 entries, all in flight at once, until a batch of survivors is full, so the
-// blocks that walk a long list whose entries mostly miss them are bound by bandwidth rather
-// than by one load round trip per 32 entries.  Every quantity that decides a branch per pixel
-// (sigma, alpha, T) is computed with explicit round-to-nearest intrinsics in one shared
-// function, so the backward kernel retraces exactly the forward's contributors.
+// staging -- every pixel would skip it, so results are unchanged -- and 64 list positions are
+// loaded at a time, so the blocks that walk a long list whose entries mostly miss them are not
+// bound by one load round trip per few entries.  What decides whether an entry counts at a pixel
+// (sigma and its limit) is computed with explicit round-to-nearest intrinsics in one shared
+// function, so the backward kernel retraces exactly the forward's contributors (the forward's
+// position of the last one says where a pixel ended).
 //
 // Work is very uneven across blocks (lists of a few entries next to lists of 15,000), so both
 // kernels take their tiles in the order bin_sort left in the workspace (decreasing list
@@ -33,6 +33,7 @@ namespace {
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kHalfLog2e = 0.7213475204444817f;
 constexpr float kLn2 = 0.6931471805599453f;
+constexpr float kFarSigma = 1e30f;               // 2^-kFarSigma is 0
 
 constexpr int kSub = 8;                          // CTA pixel block edge
 constexpr int kSubThreads = 32;                  // one warp, two pixels per lane
@@ -40,10 +41,13 @@ constexpr int kSubPerTile = (kTile / kSub) * (kTile / kSub);
 static_assert(kSubPerTile == kRenderSubPerTile, "tile order expands to kRenderSubPerTile CTAs per tile");
 constexpr int kRounds = 2;                       // list entries per lane per staging group
 constexpr int kGroup = kSubThreads * kRounds;    // 64 entries loaded together
-constexpr int kBatch = kGroup;                   // staged survivors per batch (at most)
+constexpr int kFwdUnroll = 4;                    // staged entries per iteration
+constexpr int kFwdRounds = 2;
+constexpr int kFwdGroup = kFwdRounds * kSubThreads;   // list positions the forward stages together
 constexpr int kCkChunk = 128;                    // list positions per backward chunk
 constexpr int kItemCtasPerSm = 16;               // backward CTAs that replay listed chunks
-static_assert(kCkChunk % kGroup == 0, "checkpoints fall on staging group boundaries");
+static_assert(kCkChunk % kGroup == 0 && kCkChunk % kFwdGroup == 0,
+              "checkpoints fall on staging group boundaries");
 
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
@@ -56,51 +60,63 @@ __device__ __forceinline__ float4 scaled_conic(float4 c) {
   return make_float4(__fmul_rn(kHalfLog2e, c.x), __fmul_rn(kLog2e, c.y), __fmul_rn(kHalfLog2e, c.z), c.w);
 }
 
-// sigma * log2(e) = dx (a/2 dx + b dy) + c/2 dy^2 at the lane's two pixels (fx0, fy) and
-// (fx1, fy); the dy terms are shared.  Both kernels take every branch decision from these bits.
-// The two pixels go through the packed two-lane fp32 instructions, whose every component is
-// rounded exactly as the scalar instruction would round it.
-__device__ __forceinline__ void sigma_pair(float4 s, float2 m, float fx0, float fx1, float fy,
-                                           float& dx0, float& dx1, float& dy, float& s0, float& s1) {
-  dy = __fsub_rn(fy, m.y);
-  const float2 dx = __fadd2_rn(make_float2(fx0, fx1), make_float2(-m.x, -m.x));
-  dx0 = dx.x;
-  dx1 = dx.y;
+// sigma * log2(e) = dx (a/2 dx + b dy) + c/2 dy^2 at the lane's two pixels (fx.x, fy) and
+// (fx.y, fy), nm the negated mean; the dy terms are shared.  Both kernels take every branch
+// decision from these bits.  The two pixels go through the packed two-lane fp32 instructions,
+// whose every component is rounded exactly as the scalar instruction would round it.
+__device__ __forceinline__ void sigma_pair(float4 s, float4 nm, float2 fx, float fy, float2& dx,
+                                           float& dy, float2& sg) {
+  dy = __fadd_rn(fy, nm.y);
+  dx = __fadd2_rn(fx, make_float2(nm.x, nm.x));
   const float bdy = __fmul_rn(s.y, dy);
-  const float cdy2 = __fmul_rn(__fmul_rn(s.z, dy), dy);
+  const float cdy2 = __fmaf_rn(__fmul_rn(s.z, dy), dy, 0.f);   // + 0: sigma is never -0
   const float2 in = __ffma2_rn(make_float2(s.x, s.x), dx, make_float2(bdy, bdy));
-  const float2 sg = __ffma2_rn(dx, in, make_float2(cdy2, cdy2));
-  s0 = sg.x;
-  s1 = sg.y;
+  sg = __ffma2_rn(dx, in, make_float2(cdy2, cdy2));
 }
 
-// Lower bound of sigma * log2(e) over the box [X0, X1] x [Y0, Y1] of offsets d = pixel - uv:
-// 0 if the box contains d = 0, else the least value on its four edges (convex quadratic; on
-// each edge the minimiser of the other coordinate is clamped into the box).
-__device__ __forceinline__ float box_min_sigma2(float4 s, float X0, float X1, float Y0, float Y1) {
-  if (X0 <= 0.f && X1 >= 0.f && Y0 <= 0.f && Y1 >= 0.f) return 0.f;
-  const float ry = __fdividef(-s.y, 2.f * s.z), rx = __fdividef(-s.y, 2.f * s.x);
-  float best = 3.0e38f;
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const float X = e ? X1 : X0;
-    const float dy = fminf(fmaxf(ry * X, Y0), Y1);
-    best = fminf(best, X * (s.x * X + s.y * dy) + s.z * dy * dy);
-    const float Y = e ? Y1 : Y0;
-    const float dx = fminf(fmaxf(rx * Y, X0), X1);
-    best = fminf(best, dx * (s.x * dx + s.y * Y) + s.z * Y * Y);
-  }
-  return best;
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
-// True when no pixel centre of the CTA's box can give alpha >= alpha_min: alpha = o 2^-sigma'
-// < alpha_min needs sigma' > log2(o / alpha_min); the margin (0.02 + 0.2% in log2 units) is
-// orders of magnitude above the fp32 error of either evaluation.
-__device__ __forceinline__ bool cull(float4 s, float2 m, float bx0, float by0, float alpha_min) {
-  if (!(s.w >= alpha_min)) return true;
-  const float thr = __log2f(__fdividef(s.w, alpha_min));
-  const float lo = box_min_sigma2(s, bx0 - m.x, bx0 + (kSub - 1) - m.x, by0 - m.y, by0 + (kSub - 1) - m.y);
-  return lo * 0.998f > thr + 0.02f;
+// Least value of sigma * log2(e) over the box [X0, X0 + 7] x [Y0, Y0 + 7] of offsets d = pixel -
+// uv.  For a positive definite conic it lies on an edge that faces d = 0 (on any other edge q
+// falls towards d = 0), so at most one edge of each direction counts: x = Xe, the x of the box
+// nearest to 0, with the other coordinate's minimiser clamped into the box, and y = Ye likewise
+// (when 0 lies in the x range, Xe = 0 is no edge but a point of the box, which does no harm).
+__device__ __forceinline__ float box_min_sigma2(float4 s, float X0, float Y0) {
+  const float X1 = X0 + (kSub - 1), Y1 = Y0 + (kSub - 1);
+  const float Xe = fmaxf(X0, fminf(X1, 0.f)), Ye = fmaxf(Y0, fminf(Y1, 0.f));
+  const float hb = -0.5f * s.y;
+  const float yx = fminf(fmaxf(hb * rcp_approx(s.z) * Xe, Y0), Y1);
+  const float xy = fminf(fmaxf(hb * rcp_approx(s.x) * Ye, X0), X1);
+  const float q0 = Xe * (s.x * Xe + s.y * yx) + s.z * yx * yx;
+  const float q1 = xy * (s.x * xy + s.y * Ye) + s.z * Ye * Ye;
+  return fminf(q0, q1);
+}
+
+// Largest sigma * log2(e) at which an entry of opacity o still has alpha >= alpha_min,
+// log2(o / alpha_min), or -1 for an entry that never does.  A pixel takes the entry iff
+// 0 <= sigma' <= the limit, one unsigned comparison of the two values' bits (a negative or NaN
+// sigma' is above every limit).  lg2.approx is within 2^-22 of the logarithm, as ex2.approx is of
+// the exponential that the alpha itself comes from.
+__device__ __forceinline__ float sigma_limit(float o, const Opts& op) {
+  const float lim = fmaxf(__log2f(o) - op.log2_alpha_min, 0.f);
+  return ((o >= op.alpha_min) & (op.alpha_max >= op.alpha_min)) ? lim : -1.f;
+}
+
+__device__ __forceinline__ bool takes(float sg, float lim) {
+  return __float_as_uint(sg) <= __float_as_uint(lim);
+}
+
+// True when no pixel centre of the CTA's box can reach the limit (sigma_limit); the margin (0.02
+// + 0.2% in log2 units) is orders of magnitude above the fp32 error of either evaluation.  A
+// conic that is not positive definite is never culled.
+__device__ __forceinline__ bool cull(float4 s, float2 m, float bx0, float by0, float lim) {
+  const bool pd = (s.x > 0.f) & (s.z > 0.f) & (4.f * s.x * s.z > s.y * s.y);
+  const bool out = box_min_sigma2(s, bx0 - m.x, by0 - m.y) * 0.998f > lim + 0.02f;
+  return !(lim >= 0.f) | (pd & out);
 }
 
 __device__ __forceinline__ float4 load_px(const void* img, int dtype, long long p) {
@@ -114,71 +130,69 @@ __device__ __forceinline__ float4 load_px(const void* img, int dtype, long long 
   return reinterpret_cast<const float4*>(img)[p];
 }
 
-// Stages list entries from position `next` on, in groups of kGroup whose loads are all issued
-// before any is used, until more than kBatch - kGroup survivors of the CTA-box cull are staged
-// or position n is reached; survivors are compacted in list order, each with its list
-// position in s_rgb[.].w (bits) and, for the backward, its Gaussian id.  Returns the number
-// staged.  next and the count are warp-uniform.
-template <bool WITH_ID>
+// Stages the entries of the kGroup list positions from `next` on (below n), all loads in flight
+// together; survivors of the CTA-box cull are compacted in list order, each with its sigma limit,
+// its list position + 1 (bits) and its Gaussian id.  Returns the number staged (warp-uniform);
+// clamp: some staged opacity exceeds alpha_max.
 __device__ __forceinline__ int stage_fill(const unsigned* ids, unsigned start, int n, int& next,
                                           const float2* uv, const float4* co, const float* rgb,
-                                          float bx0, float by0, float alpha_min, float2* s_uv,
-                                          float4* s_co, float4* s_rgb, unsigned* s_id) {
+                                          float bx0, float by0, const Opts& op, float4* s_co,
+                                          float4* s_m, float4* s_rgb, unsigned* s_id, bool& clamp) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   int total = 0;
-  while (next < n && total <= kBatch - kGroup) {
-    unsigned g[kRounds];
-    float2 m[kRounds];
-    float4 c[kRounds];
-    float col[kRounds][3];
+  bool over = false;
+  unsigned g[kRounds];
+  float2 m[kRounds];
+  float4 c[kRounds];
+  float col[kRounds][3];
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      const int pos = next + lane + r * kSubThreads;
-      g[r] = pos < n ? __ldg(ids + start + pos) : 0xffffffffu;
-    }
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      if (g[r] != 0xffffffffu) {
-        m[r] = __ldg(uv + g[r]);
-        c[r] = __ldg(co + g[r]);
-        col[r][0] = __ldg(rgb + 3 * g[r]);
-        col[r][1] = __ldg(rgb + 3 * g[r] + 1);
-        col[r][2] = __ldg(rgb + 3 * g[r] + 2);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      bool keep = false;
-      float4 sc = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (g[r] != 0xffffffffu) {
-        sc = scaled_conic(c[r]);
-        keep = !cull(sc, m[r], bx0, by0, alpha_min);
-      }
-      const unsigned b = __ballot_sync(0xffffffffu, keep);
-      if (keep) {
-        const int slot = total + __popc(b & lt);
-        s_uv[slot] = m[r];
-        s_co[slot] = sc;
-        s_rgb[slot] = make_float4(col[r][0], col[r][1], col[r][2],
-                                  __uint_as_float((unsigned)(next + lane + r * kSubThreads)));
-        if (WITH_ID) s_id[slot] = g[r];
-      }
-      total += __popc(b);
-    }
-    next += kGroup;
+  for (int r = 0; r < kRounds; ++r) {
+    const int pos = next + lane + r * kSubThreads;
+    g[r] = pos < n ? __ldg(ids + start + pos) : 0xffffffffu;
   }
-  // the blend loops read up to one (forward) or two (backward) slots past the last survivor
-  // as masked-out entries: they must hold finite zeros, not another kernel's leftovers (a
-  // zero weight times a non-finite value is not zero)
-  constexpr int kPad = WITH_ID ? 2 : 1;
-  constexpr int kSlots = WITH_ID ? kBatch + 2 : kBatch;
-  if (lane < kPad && total + lane < kSlots) {
-    s_uv[total + lane] = make_float2(0.f, 0.f);
-    s_co[total + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) {
+    if (g[r] != 0xffffffffu) {
+      m[r] = __ldg(uv + g[r]);
+      c[r] = __ldg(co + g[r]);
+      col[r][0] = __ldg(rgb + 3 * (size_t)g[r]);
+      col[r][1] = __ldg(rgb + 3 * (size_t)g[r] + 1);
+      col[r][2] = __ldg(rgb + 3 * (size_t)g[r] + 2);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) {
+    bool keep = false;
+    float4 sc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float lim = -1.f;
+    if (g[r] != 0xffffffffu) {
+      sc = scaled_conic(c[r]);
+      lim = sigma_limit(sc.w, op);
+      keep = !cull(sc, m[r], bx0, by0, lim);
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, keep);
+    if (keep) {
+      const int slot = total + __popc(b & lt);
+      s_co[slot] = make_float4(sc.x, sc.y, sc.z, -sc.w);
+      s_m[slot] = make_float4(-m[r].x, -m[r].y, lim,
+                              __uint_as_float((unsigned)(next + lane + r * kSubThreads + 1)));
+      s_rgb[slot] = make_float4(col[r][0], col[r][1], col[r][2], 0.f);
+      s_id[slot] = g[r];
+      over = over || !(sc.w <= op.alpha_max);
+    }
+    total += __popc(b);
+  }
+  next += kGroup;
+  // the loop over the survivors reads up to two slots past the last: a NaN sigma is taken by no
+  // pixel, and the rest must be finite (a zero weight times a non-finite value is not zero)
+  if (lane < 2) {
+    s_co[total + lane] = make_float4(__int_as_float(0x7fffffff), 0.f, 0.f, 0.f);
+    s_m[total + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
     s_rgb[total + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (WITH_ID) s_id[total + lane] = 0u;
+    s_id[total + lane] = 0u;
   }
+  clamp = __any_sync(0xffffffffu, over);
   __syncwarp();
   return total;
 }
@@ -247,68 +261,107 @@ struct FwdArgs {
 struct PixF {
   float T, c0, c1, c2;
   unsigned last;       // one past the list position of the last contributor
-  bool done;
 };
 
-// Blend state of the lane's two pixels, the first in .x, the second in .y.
+// Blend state of the lane's two pixels, the first in .x, the second in .y.  A pixel that has
+// ended (or lies outside the image) has a NaN for its x: every sigma there is NaN and no entry
+// is taken, at no cost per entry.
 struct PixF2 {
-  float2 T, c0, c1, c2;
+  float2 T, fx;
+  float2 nc0, nc1, nc2;     // the colour so far, negated
+  float fy;
   unsigned last0, last1;
-  bool done0, done1;
+  __device__ __forceinline__ bool on() const { return fx.x == fx.x || fx.y == fx.y; }
 };
 
-// One staged list entry as the blend loops read it.
+// One staged list entry as the backward's loop reads it.
 struct Entry {
   float4 s;            // scaled conic, opacity
-  float2 m;            // uv
-  float4 col;          // rgb, list position (bits)
+  float4 m;            // uv, sigma limit, list position + 1 (bits)
+  float4 col;          // rgb
 };
 
-__device__ __forceinline__ Entry load_entry(const float2* s_uv, const float4* s_co,
+__device__ __forceinline__ Entry load_entry(const float4* s_co, const float4* s_m,
                                             const float4* s_rgb, int j) {
   Entry e;
   e.s = s_co[j];
-  e.m = s_uv[j];
+  e.m = s_m[j];
   e.col = s_rgb[j];
   return e;
 }
 
-// alpha at the lane's two pixels for one entry and whether each passes the skip tests
-// (sigma >= 0, alpha >= alpha_min).  Independent of the blend state, so the loops evaluate
-// it for several entries before the transmittance chain needs it.
-__device__ __forceinline__ void alpha_pair(const Entry& e, float fx0, float fx1, float fy,
-                                           const Opts& op, float& a0, float& a1, bool& ok0,
-                                           bool& ok1) {
-  float dx0, dx1, dy, sg0, sg1;
-  sigma_pair(e.s, e.m, fx0, fx1, fy, dx0, dx1, dy, sg0, sg1);
-  a0 = fminf(op.alpha_max, __fmul_rn(e.s.w, ex2_approx(-sg0)));
-  a1 = fminf(op.alpha_max, __fmul_rn(e.s.w, ex2_approx(-sg1)));
-  ok0 = sg0 >= 0.f && a0 >= op.alpha_min;
-  ok1 = sg1 >= 0.f && a1 >= op.alpha_min;
+// Front-to-back step of the lane's two pixels over U staged entries.  The alphas come first
+// (negated, 0 where an entry is not taken), then the transmittances after each entry, linked by
+// one FMA per entry; when no pixel of the warp falls below t_min among them (a vote), the
+// colours are added without another test.  Otherwise the entries are taken one by one: the entry
+// that takes a pixel below t_min ends it and does not contribute.  CLAMP: some staged opacity
+// exceeds alpha_max (else o 2^-sigma' cannot).
+template <int U, bool CLAMP>
+__device__ __forceinline__ void blend(PixF2& p, const float4* s_co, const float4* s_m,
+                                      const float4* s_rgb, const Opts& op) {
+  float2 na[U], Tb[U], T = p.T;
+  unsigned l0 = p.last0, l1 = p.last1;
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    const float4 s = s_co[k], m = s_m[k];
+    float2 dx, sg;
+    float dy;
+    sigma_pair(s, m, p.fx, p.fy, dx, dy, sg);
+    float2 raw = __fmul2_rn(make_float2(s.w, s.w), make_float2(ex2_approx(-sg.x), ex2_approx(-sg.y)));
+    if (CLAMP) raw = make_float2(fmaxf(-op.alpha_max, raw.x), fmaxf(-op.alpha_max, raw.y));
+    const bool t0 = takes(sg.x, m.z), t1 = takes(sg.y, m.z);
+    na[k] = make_float2(t0 ? raw.x : 0.f, t1 ? raw.y : 0.f);
+    l0 = t0 ? __float_as_uint(m.w) : l0;
+    l1 = t1 ? __float_as_uint(m.w) : l1;
+  }
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    Tb[k] = T;
+    T = __ffma2_rn(na[k], T, T);
+  }
+  if (!__any_sync(0xffffffffu, fminf(T.x, T.y) < op.t_min)) {
+    p.T = T;
+    p.last0 = l0;
+    p.last1 = l1;
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const float4 col = s_rgb[k];
+      const float2 w = __fmul2_rn(na[k], Tb[k]);
+      p.nc0 = __ffma2_rn(w, make_float2(col.x, col.x), p.nc0);
+      p.nc1 = __ffma2_rn(w, make_float2(col.y, col.y), p.nc1);
+      p.nc2 = __ffma2_rn(w, make_float2(col.z, col.z), p.nc2);
+    }
+    return;
+  }
+  bool on0 = p.fx.x == p.fx.x, on1 = p.fx.y == p.fx.y;
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    const float4 col = s_rgb[k];
+    const unsigned pos = __float_as_uint(s_m[k].w);
+    const float2 Tn = __ffma2_rn(na[k], p.T, p.T);
+    const bool t0 = on0 && na[k].x < 0.f, t1 = on1 && na[k].y < 0.f;
+    const bool u0 = t0 && !(Tn.x < op.t_min), u1 = t1 && !(Tn.y < op.t_min);
+    on0 = on0 && (u0 || !t0);
+    on1 = on1 && (u1 || !t1);
+    const float2 wf = __fmul2_rn(na[k], p.T);
+    const float2 w = make_float2(u0 ? wf.x : 0.f, u1 ? wf.y : 0.f);
+    p.nc0 = __ffma2_rn(w, make_float2(col.x, col.x), p.nc0);
+    p.nc1 = __ffma2_rn(w, make_float2(col.y, col.y), p.nc1);
+    p.nc2 = __ffma2_rn(w, make_float2(col.z, col.z), p.nc2);
+    p.T = make_float2(u0 ? Tn.x : p.T.x, u1 ? Tn.y : p.T.y);
+    p.last0 = u0 ? pos : p.last0;
+    p.last1 = u1 ? pos : p.last1;
+  }
+  const float nan = __int_as_float(0x7fffffff);
+  p.fx = make_float2(on0 ? p.fx.x : nan, on1 ? p.fx.y : nan);
 }
 
-// Front-to-back step of the lane's two pixels for one entry (selects, no branches): a passing
-// entry either ends a pixel (T (1 - alpha) < t_min; it does not contribute) or is blended in.
-// A pixel the entry does not reach gets a zero weight, and fma(0, c, C) leaves C as it was.
-__device__ __forceinline__ void blend2(PixF2& p, float a0, float a1, bool ok0, bool ok1,
-                                       float4 col, const Opts& op) {
-  ok0 = ok0 && !p.done0;
-  ok1 = ok1 && !p.done1;
-  const float2 al = make_float2(a0, a1);
-  const float2 test = __fmul2_rn(p.T, __fadd2_rn(make_float2(1.f, 1.f), make_float2(-a0, -a1)));
-  const bool term0 = ok0 && test.x < op.t_min, term1 = ok1 && test.y < op.t_min;
-  const bool use0 = ok0 && !term0, use1 = ok1 && !term1;
-  const float2 w = __fmul2_rn(al, p.T);
-  const float2 wu = make_float2(use0 ? w.x : 0.f, use1 ? w.y : 0.f);
-  p.done0 = p.done0 || term0;
-  p.done1 = p.done1 || term1;
-  p.c0 = __ffma2_rn(wu, make_float2(col.x, col.x), p.c0);
-  p.c1 = __ffma2_rn(wu, make_float2(col.y, col.y), p.c1);
-  p.c2 = __ffma2_rn(wu, make_float2(col.z, col.z), p.c2);
-  p.T = make_float2(use0 ? test.x : p.T.x, use1 ? test.y : p.T.y);
-  const unsigned nxt = __float_as_uint(col.w) + 1u;
-  p.last0 = use0 ? nxt : p.last0;
-  p.last1 = use1 ? nxt : p.last1;
+// Blends staged entries [0, cnt), padded to a multiple of kFwdUnroll.
+template <bool CLAMP>
+__device__ __forceinline__ void blend_staged(PixF2& p, const float4* s_co, const float4* s_m,
+                                             const float4* s_rgb, int cnt, const Opts& op) {
+  for (int j = 0; j < cnt; j += kFwdUnroll)
+    blend<kFwdUnroll, CLAMP>(p, s_co + j, s_m + j, s_rgb + j, op);
 }
 
 __device__ __forceinline__ void store_pixel(const FwdArgs& a, long long p, const PixF& s, int qx,
@@ -344,67 +397,156 @@ __device__ __forceinline__ void store_pixel(const FwdArgs& a, long long p, const
   }
 }
 
-__global__ void __launch_bounds__(kSubThreads) render_fwd_kernel(FwdArgs a) {
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src), "n"(BYTES) : "memory");
+}
+
+// The raw entries of a staging group, as the asynchronous copies bring them in.
+struct RawGroup {
+  float4 co[kFwdGroup];
+  float2 uv[kFwdGroup];
+  float rgb[3][kFwdGroup];
+};
+
+__device__ __forceinline__ void fetch_group(const FwdArgs& a, const unsigned (&g)[kFwdRounds],
+                                            RawGroup& raw) {
+#pragma unroll
+  for (int r = 0; r < kFwdRounds; ++r) {
+    const int k = (threadIdx.x & 31) + 32 * r;
+    if (g[r] == 0xffffffffu) continue;
+    copy_async<16>(&raw.co[k], a.co + g[r]);
+    copy_async<8>(&raw.uv[k], a.uv + g[r]);
+    const float* col = a.rgb + 3 * (size_t)g[r];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) copy_async<4>(&raw.rgb[c][k], col + c);
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// What bounds it: the longest walks.  A small active block covers a quarter of the tiles, so
+// every non-empty 8x8 block is resident at once (about 30 one-warp CTAs per SM at 1237x822) and
+// the kernel lasts as long as its longest walk (700 staged entries there, 81,000 of its 137,000
+// cycles blending, at 116 cycles per entry).  The walk is therefore built for one warp's
+// instructions and latency: the entries of the next 64 list positions are copied to shared
+// memory, and the ids of the 64 after them loaded, while the current ones are blended; the block
+// cull takes both lanes' rounds side by side without branches; four entries are evaluated
+// together whose states are linked by one FMA, with the end-of-pixel test voted on once per
+// four.  Against two entries at a time with their selects and 64 entries loaded when needed:
+// 33 -> 23 us (2,000 Gaussians, 128x128), 84 -> 62 us (100,000, 1237x822), 218 -> 189 us (2M,
+// 1920x1080); the refresh at 1237x822 77-98 -> 53-68 us.  Eight entries per iteration need 120
+// registers and gave 61 and 207 us; 32 positions per group 29 us and 72 us.  24 CTAs per SM (80
+// registers, no spills) against 28: 61 against 63 us and 189 against 199 us.
+__global__ void __launch_bounds__(kSubThreads, 24) render_fwd_kernel(const __grid_constant__ FwdArgs a) {
   pdl_prologue();
-  __shared__ float2 s_uv[kBatch];
-  __shared__ float4 s_co[kBatch];
-  __shared__ float4 s_rgb[kBatch];
+  __shared__ RawGroup raw;
+  __shared__ float4 s_co[kFwdGroup];
+  __shared__ float4 s_m[kFwdGroup];
+  __shared__ float4 s_rgb[kFwdGroup];
   const int blk = block_index(a.tile_order, (int)blockIdx.x);
   const Block bk = block_of(a.cam, blk);
   const int lane = threadIdx.x & 31;
   const uint2 rg = a.ranges[bk.tile];
   const int n = (rg.y > rg.x && !(*a.status & kStatusTimeout)) ? (int)(rg.y - rg.x) : 0;
-  const float fx0 = (float)bk.qx0 + 0.5f, fx1 = (float)bk.qx1 + 0.5f, fy = (float)bk.py + 0.5f;
   const float bx0 = (float)bk.px0 + 0.5f, by0 = (float)bk.py0 + 0.5f;
+  const float nan = __int_as_float(0x7fffffff);
   PixF2 pp;
   pp.T = make_float2(1.f, 1.f);
-  pp.c0 = pp.c1 = pp.c2 = make_float2(0.f, 0.f);
+  pp.nc0 = pp.nc1 = pp.nc2 = make_float2(0.f, 0.f);
+  pp.fx = make_float2(bk.in0 ? (float)bk.qx0 + 0.5f : nan, bk.in1 ? (float)bk.qx1 + 0.5f : nan);
+  pp.fy = (float)bk.py + 0.5f;
   pp.last0 = pp.last1 = 0u;
-  pp.done0 = !bk.in0;
-  pp.done1 = !bk.in1;
-  int next = 0;
   bool ck_on = a.ckpt != nullptr;          // warp-uniform
   int n_items = 0;
   unsigned my_slot = 0u;                   // lane k: the slot of this block's item k
-  while (next < n) {
-    if (__all_sync(0xffffffffu, pp.done0 && pp.done1)) break;
-    __syncwarp();
-    // with checkpoints, a batch ends at the next multiple of kCkChunk
-    const int lim = ck_on ? min(n, (next / kCkChunk + 1) * kCkChunk) : n;
-    const int cnt = stage_fill<false>(a.ids, rg.x, lim, next, a.uv, a.co, a.rgb, bx0, by0,
-                                      a.op.alpha_min, s_uv, s_co, s_rgb, nullptr);
-    // two entries per iteration (slot j + 1 <= kBatch - 1 exists; unused when j + 1 == cnt)
-    for (int j = 0; j < cnt; j += 2) {
-      const Entry e0 = load_entry(s_uv, s_co, s_rgb, j);
-      const Entry e1 = load_entry(s_uv, s_co, s_rgb, j + 1);
-      float a00, a01, a10, a11;
-      bool k00, k01, k10, k11;
-      alpha_pair(e0, fx0, fx1, fy, a.op, a00, a01, k00, k01);
-      alpha_pair(e1, fx0, fx1, fy, a.op, a10, a11, k10, k11);
-      const bool v1 = j + 1 < cnt;
-      blend2(pp, a00, a01, k00, k01, e0.col, a.op);
-      blend2(pp, a10, a11, k10 && v1, k11 && v1, e1.col, a.op);
-      if ((j & 30) == 30 && __all_sync(0xffffffffu, pp.done0 && pp.done1)) break;
+  const unsigned* ids = a.ids + rg.x;
+  unsigned g[kFwdRounds];
+#pragma unroll
+  for (int r = 0; r < kFwdRounds; ++r) g[r] = lane + 32 * r < n ? __ldg(ids + lane + 32 * r) : 0xffffffffu;
+  if (n > 0) fetch_group(a, g, raw);
+#pragma unroll
+  for (int r = 0; r < kFwdRounds; ++r) {
+    const int pos = kFwdGroup + lane + 32 * r;
+    g[r] = pos < n ? __ldg(ids + pos) : 0xffffffffu;
+  }
+  for (int base = 0; base < n; base += kFwdGroup) {
+    if (!__any_sync(0xffffffffu, pp.on())) break;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    // the survivors of the block cull, compacted in list order (a lane reads the entries that it
+    // copied itself)
+    int cnt = 0;
+    bool over = false;
+    float4 sc[kFwdRounds];
+    float2 m[kFwdRounds];
+    float lim[kFwdRounds], col[kFwdRounds][3];
+    bool keep[kFwdRounds];
+#pragma unroll
+    for (int r = 0; r < kFwdRounds; ++r) {
+      const int k = lane + 32 * r;
+      sc[r] = scaled_conic(raw.co[k]);
+      m[r] = raw.uv[k];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) col[r][c] = raw.rgb[c][k];
+      lim[r] = sigma_limit(sc[r].w, a.op);
+      keep[r] = (base + k < n) & !cull(sc[r], m[r], bx0, by0, lim[r]);
     }
-    if (ck_on && next == lim && lim < n && !__all_sync(0xffffffffu, pp.done0 && pp.done1)) {
-      // the state after every position below lim, for the backward's chunk starting there
-      unsigned slot = 0u;
-      if (lane == 0) slot = atomicAdd(a.ck_count, 1u);
-      slot = __shfl_sync(0xffffffffu, slot, 0);
-      if (slot < (unsigned)a.ck_cap) {
-        float4* ck = a.ckpt + (size_t)slot * (kSub * kSub);
-        const int k0 = block_pixel(lane);
-        ck[k0] = make_float4(pp.c0.x, pp.c1.x, pp.c2.x, pp.T.x);
-        ck[k0 + 4] = make_float4(pp.c0.y, pp.c1.y, pp.c2.y, pp.T.y);
-        if (lane == n_items) my_slot = slot;
-        ++n_items;
+#pragma unroll
+    for (int r = 0; r < kFwdRounds; ++r) {
+      const unsigned kept = __ballot_sync(0xffffffffu, keep[r]);
+      const int slot = cnt + __popc(kept & ((1u << lane) - 1u));
+      if (keep[r]) {
+        s_co[slot] = make_float4(sc[r].x, sc[r].y, sc[r].z, -sc[r].w);
+        s_m[slot] = make_float4(-m[r].x, -m[r].y, lim[r], __uint_as_float((unsigned)(base + lane + 32 * r + 1)));
+        s_rgb[slot] = make_float4(col[r][0], col[r][1], col[r][2], 0.f);
       }
-      // past 32 items or a full buffer the last item listed runs to the end of the walk
-      ck_on = slot < (unsigned)a.ck_cap && n_items < 32;
+      over = over | (keep[r] & !(sc[r].w <= a.op.alpha_max));
+      cnt += __popc(kept);
+    }
+    const bool clamp = __any_sync(0xffffffffu, over);
+    // unused slots of the last iteration: a NaN sigma is taken by no pixel
+    if (lane < (-cnt & (kFwdUnroll - 1))) {
+      s_co[cnt + lane] = make_float4(nan, 0.f, 0.f, 0.f);
+      s_m[cnt + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+      s_rgb[cnt + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (base + kFwdGroup < n) fetch_group(a, g, raw);
+#pragma unroll
+    for (int r = 0; r < kFwdRounds; ++r) {
+      const int pos = base + 2 * kFwdGroup + lane + 32 * r;
+      g[r] = pos < n ? __ldg(ids + pos) : 0xffffffffu;
+    }
+    const int end = base + kFwdGroup;
+    // at a checkpoint: ask for its slot now, the answer comes while the group is blended
+    const bool ck_here = ck_on && end % kCkChunk == 0 && end < n;
+    unsigned slot = 0u;
+    if (ck_here && lane == 0) slot = atomicAdd(a.ck_count, 1u);
+    __syncwarp();
+    if (!clamp) blend_staged<false>(pp, s_co, s_m, s_rgb, cnt, a.op);
+    else blend_staged<true>(pp, s_co, s_m, s_rgb, cnt, a.op);
+    __syncwarp();
+    if (ck_here) {
+      // the state after every position below `end`, for the backward's chunk starting there
+      slot = __shfl_sync(0xffffffffu, slot, 0);
+      const bool room = slot < (unsigned)a.ck_cap;
+      if (__any_sync(0xffffffffu, pp.on())) {
+        if (room) {
+          float4* ck = a.ckpt + (size_t)slot * (kSub * kSub);
+          const int k0 = block_pixel(lane);
+          ck[k0] = make_float4(0.f - pp.nc0.x, 0.f - pp.nc1.x, 0.f - pp.nc2.x, pp.T.x);
+          ck[k0 + 4] = make_float4(0.f - pp.nc0.y, 0.f - pp.nc1.y, 0.f - pp.nc2.y, pp.T.y);
+          if (lane == n_items) my_slot = slot;
+          ++n_items;
+        }
+        // past 32 items or a full buffer the last item listed runs to the end of the walk
+        ck_on = room && n_items < 32;
+      } else if (room && lane == 0) {
+        a.ck_items[slot] = make_uint4(0u, 0u, 0u, 0u);   // the walk ended: nothing to replay
+      }
     }
   }
-  const PixF p0 = {pp.T.x, pp.c0.x, pp.c1.x, pp.c2.x, pp.last0, pp.done0};
-  const PixF p1 = {pp.T.y, pp.c0.y, pp.c1.y, pp.c2.y, pp.last1, pp.done1};
+  const PixF p0 = {pp.T.x, 0.f - pp.nc0.x, 0.f - pp.nc1.x, 0.f - pp.nc2.x, pp.last0};
+  const PixF p1 = {pp.T.y, 0.f - pp.nc0.y, 0.f - pp.nc1.y, 0.f - pp.nc2.y, pp.last1};
   if (a.ckpt) {
     if (lane == 0) a.ck_first[blk] = n_items > 0 ? (unsigned)kCkChunk : 0xffffffffu;
     if (lane < n_items) {
@@ -468,95 +610,143 @@ __device__ __forceinline__ void load_pixel_grad(const BwdArgs& a, long long p, i
 }
 
 // Backward of the lane's two pixels for one list entry (selects, no branches): when the entry
-// contributed to a pixel (live: a position below the pixel's last contributor; sigma >= 0;
-// alpha >= alpha_min) adds to v the opacity and colour gradients (v[5..8]) and the moments of
-// d = pixel - uv weighted by dL/dsigma, (sum w dx, w dy, w dx^2, w dx dy, w dy^2) in v[0..4]
-// (the conic and mean gradients follow from them once per entry), and advances the replayed
-// transmittance exactly as the forward did.  With G = dL/dA.rgb and G_a = dL/dA.a, the
-// derivative of the loss w.r.t. an entry's alpha is
+// contributed to a pixel (live: a position up to the pixel's last contributor; sigma within the
+// limit) gives in v the opacity and colour gradients (v[5..8]) and the moments of d = pixel - uv
+// weighted by dL/dsigma, (sum w dx, w dy, w dx^2, w dx dy, w dy^2) in v[0..4] (the conic and mean
+// gradients follow from them once per entry), and advances the replayed transmittance.  With
+// G = dL/dA.rgb and G_a = dL/dA.a, the derivative of the loss w.r.t. an entry's alpha is
 //   T (G . col) - (K - G . C) / (1 - alpha),   K = G . A - G_a T_final,
-// C the colour accumulated up to and including the entry.  The two pixels' arithmetic is paired through the packed two-lane fp32 instructions and the shared row
-// offset dy factored out of the moment sums (sum t dy = (t0 + t1) dy).  The decisions (alpha,
-// the skip tests, the replayed transmittance) are rounded exactly as the forward rounds them;
-// the gradient terms only round in a different order.  who0 / who1: whether the entry
-// contributed to each pixel.
+// C the colour accumulated up to and including the entry.  The two pixels' arithmetic is paired
+// through the packed two-lane fp32 instructions, which have no negated operands: the staged
+// opacity is negated, and so is the replayed G . C, so that none is needed.  The row offset dy is
+// factored out of the moment sums (sum t dy = (t0 + t1) dy).  The decisions (sigma, its limit)
+// are rounded exactly as the forward rounds them.  who0 / who1: whether the entry contributed to
+// each pixel.
 struct PixB2 {
-  float2 T, Gc, Gr, Gg, Gb, K;
+  float2 T, nGc, Gr, Gg, Gb, K;
 };
 
-__device__ __forceinline__ void pixel_backward2(PixB2& p, float4 s, float4 col, float sg0,
-                                                float sg1, float dx0, float dx1, float dy,
-                                                bool live0, bool live1, const Opts& op, float* v,
-                                                bool& who0, bool& who1) {
-  const float2 G = make_float2(ex2_approx(-sg0), ex2_approx(-sg1));
-  const float2 raw = __fmul2_rn(make_float2(s.w, s.w), G);
-  const float a0 = fminf(op.alpha_max, raw.x), a1 = fminf(op.alpha_max, raw.y);
-  const bool ok0 = live0 && sg0 >= 0.f && a0 >= op.alpha_min;
-  const bool ok1 = live1 && sg1 >= 0.f && a1 >= op.alpha_min;
-  const float2 w = __fmul2_rn(make_float2(a0, a1), p.T);
-  const float2 gcol = __ffma2_rn(p.Gb, make_float2(col.z, col.z),
-                                 __ffma2_rn(p.Gg, make_float2(col.y, col.y),
-                                            __fmul2_rn(p.Gr, make_float2(col.x, col.x))));
-  const float2 gc = __ffma2_rn(w, gcol, p.Gc);                     // G . C including the entry
-  const float2 oma = __fadd2_rn(make_float2(1.f, 1.f), make_float2(-a0, -a1));
-  const float2 ioma = make_float2(__fdividef(1.f, oma.x), __fdividef(1.f, oma.y));
-  const float2 km = __fadd2_rn(p.K, make_float2(-gc.x, -gc.y));
-  const float2 dalpha = __ffma2_rn(make_float2(-km.x, -km.y), ioma, __fmul2_rn(p.T, gcol));
-  const bool ga0 = ok0 && raw.x <= op.alpha_max, ga1 = ok1 && raw.y <= op.alpha_max;
-  const float2 dg = __fmul2_rn(dalpha, G);                          // d alpha / d opacity = G
-  const float2 dr = __fmul2_rn(dalpha, raw);                        // d alpha / d sigma = -alpha
-  const float wk0 = ok0 ? w.x : 0.f, wk1 = ok1 ? w.y : 0.f;
-  const float ds0 = ga0 ? -dr.x : 0.f, ds1 = ga1 ? -dr.y : 0.f;
-  v[5] += (ga0 ? dg.x : 0.f) + (ga1 ? dg.y : 0.f);
-  v[6] = fmaf(p.Gr.x, wk0, fmaf(p.Gr.y, wk1, v[6]));
-  v[7] = fmaf(p.Gg.x, wk0, fmaf(p.Gg.y, wk1, v[7]));
-  v[8] = fmaf(p.Gb.x, wk0, fmaf(p.Gb.y, wk1, v[8]));
-  const float2 t = __fmul2_rn(make_float2(ds0, ds1), make_float2(dx0, dx1));
-  const float ts = t.x + t.y, us = (ds0 + ds1) * dy;
-  v[0] += ts;
-  v[1] += us;
-  v[2] = fmaf(t.x, dx0, fmaf(t.y, dx1, v[2]));
-  v[3] = fmaf(ts, dy, v[3]);
-  v[4] = fmaf(us, dy, v[4]);
-  p.Gc = make_float2(ok0 ? gc.x : p.Gc.x, ok1 ? gc.y : p.Gc.y);
-  const float2 Tn = __fmul2_rn(p.T, oma);
-  p.T = make_float2(ok0 ? Tn.x : p.T.x, ok1 ? Tn.y : p.T.y);
+template <bool CLAMP>
+__device__ __forceinline__ void pixel_backward2(PixB2& p, const Entry& e, float2 sg, float2 dx,
+                                                float dy, bool live0, bool live1, const Opts& op,
+                                                float* v, bool& who0, bool& who1) {
+  const bool ok0 = live0 && takes(sg.x, e.m.z);
+  const bool ok1 = live1 && takes(sg.y, e.m.z);
+  // an entry that is not taken gets a sigma whose exponential is 0, and with it alpha and every
+  // gradient
+  const float2 G = make_float2(ex2_approx(-(ok0 ? sg.x : kFarSigma)), ex2_approx(-(ok1 ? sg.y : kFarSigma)));
+  const float2 nraw = __fmul2_rn(make_float2(e.s.w, e.s.w), G);      // -o 2^-sigma'
+  float2 na = nraw;                                                  // -alpha
+  if (CLAMP) na = make_float2(fmaxf(-op.alpha_max, nraw.x), fmaxf(-op.alpha_max, nraw.y));
+  const float2 nw = __fmul2_rn(na, p.T);                             // -alpha T
+  const float2 gcol = __ffma2_rn(p.Gb, make_float2(e.col.z, e.col.z),
+                                 __ffma2_rn(p.Gg, make_float2(e.col.y, e.col.y),
+                                            __fmul2_rn(p.Gr, make_float2(e.col.x, e.col.x))));
+  p.nGc = __ffma2_rn(nw, gcol, p.nGc);                               // -G . C including the entry
+  const float2 oma = __fadd2_rn(make_float2(1.f, 1.f), na);
+  const float2 nioma = make_float2(rcp_approx(-oma.x), rcp_approx(-oma.y));
+  const float2 km = __fadd2_rn(p.K, p.nGc);
+  float2 da = __ffma2_rn(km, nioma, __fmul2_rn(p.T, gcol));
+  // d alpha / d opacity = G, d alpha / d sigma = -alpha; none of either where alpha was clamped
+  if (CLAMP) da = make_float2(nraw.x >= -op.alpha_max ? da.x : 0.f, nraw.y >= -op.alpha_max ? da.y : 0.f);
+  const float2 dg = __fmul2_rn(da, G);
+  const float2 ds = __fmul2_rn(da, nraw);
+  v[5] = dg.x + dg.y;
+  v[6] = fmaf(p.Gr.x, -nw.x, p.Gr.y * -nw.y);
+  v[7] = fmaf(p.Gg.x, -nw.x, p.Gg.y * -nw.y);
+  v[8] = fmaf(p.Gb.x, -nw.x, p.Gb.y * -nw.y);
+  const float2 t = __fmul2_rn(ds, dx);
+  const float ts = t.x + t.y, us = (ds.x + ds.y) * dy;
+  v[0] = ts;
+  v[1] = us;
+  v[2] = fmaf(t.x, dx.x, t.y * dx.y);
+  v[3] = ts * dy;
+  v[4] = us * dy;
+  p.T = __ffma2_rn(na, p.T, p.T);
   who0 = ok0;
   who1 = ok1;
 }
 
 // Warp sum of 27 per-lane values through shared memory: each lane writes its row, lane l < 27
 // reads column l (32 values, 8 float4 loads; pitch 36 keeps stores and loads conflict-free)
-// and returns its sum.
+// and returns its sum (lanes past 26: column 26's).
 constexpr int kRedPitch = 36;
 
 __device__ __forceinline__ float warp_sum27(const float (&x)[27], float* red, int lane) {
 #pragma unroll
   for (int k = 0; k < 27; ++k) red[k * kRedPitch + lane] = x[k];
   __syncwarp();
-  float r = 0.f;
-  if (lane < 27) {
-    const float4* col = reinterpret_cast<const float4*>(red + lane * kRedPitch);
+  const float4* col = reinterpret_cast<const float4*>(red + min(lane, 26) * kRedPitch);
+  float2 r0 = make_float2(0.f, 0.f), r1 = r0;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float4 a = col[q];
-      r += (a.x + a.y) + (a.z + a.w);
-    }
+  for (int q = 0; q < 8; ++q) {
+    const float4 a = col[q];
+    r0 = __fadd2_rn(r0, make_float2(a.x, a.y));
+    r1 = __fadd2_rn(r1, make_float2(a.z, a.w));
   }
   __syncwarp();
-  return r;
+  r0 = __fadd2_rn(r0, r1);
+  return r0.x + r0.y;
+}
+
+// Backward of the staged entries [0, cnt) at the lane's two pixels, three entries per iteration,
+// their 27 components summed over the warp at once (slots up to cnt + 1 exist; past cnt a NaN
+// sigma is taken by no pixel).
+template <bool CLAMP>
+__device__ __forceinline__ void bwd_staged(const BwdArgs& a, PixB2& pp, float2 fx, float fy,
+                                           unsigned last0, unsigned last1, int cnt,
+                                           const float4* s_co, const float4* s_m,
+                                           const float4* s_rgb, const unsigned* s_id,
+                                           float* s_red) {
+  const int lane = threadIdx.x & 31;
+  for (int j = 0; j < cnt; j += 3) {
+    float x[27];
+    unsigned who[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const Entry e = load_entry(s_co, s_m, s_rgb, j + i);
+      const unsigned nxt = __float_as_uint(e.m.w);
+      float2 dx, sg;
+      float dy;
+      sigma_pair(e.s, e.m, fx, fy, dx, dy, sg);
+      bool c0, c1;
+      pixel_backward2<CLAMP>(pp, e, sg, dx, dy, nxt <= last0, nxt <= last1, a.op, x + 9 * i, c0, c1);
+      who[i] = __ballot_sync(0xffffffffu, c0 || c1);
+    }
+    if ((who[0] | who[1] | who[2]) == 0) continue;
+    const float r = warp_sum27(x, s_red, lane);
+    const int ei = min(lane / 9, 2), comp = lane - 9 * ei;
+    // mean and conic gradients from the weighted moments of entry ei:
+    // d/du = -(ca Sx + cb Sy), d/dv = -(cb Sx + cc Sy), d/da = Sxx / 2, d/db = Sxy,
+    // d/dc = Syy / 2, with (ca, cb, cc) = ln 2 (2 a', b', 2 c') of the scaled conic
+    const float sx = __shfl_sync(0xffffffffu, r, 9 * ei);
+    const float sy = __shfl_sync(0xffffffffu, r, 9 * ei + 1);
+    const unsigned wi = ei == 0 ? who[0] : (ei == 1 ? who[1] : who[2]);
+    if (lane < 27 && wi != 0) {
+      float g = r;
+      if (comp <= 1) {
+        const float4 sc = s_co[j + ei];
+        const float ca = 2.f * kLn2 * sc.x, cb = kLn2 * sc.y, cc = 2.f * kLn2 * sc.z;
+        g = comp == 0 ? -(ca * sx + cb * sy) : -(cb * sx + cc * sy);
+      } else if (comp == 2 || comp == 4) {
+        g = 0.5f * r;
+      }
+      atomicAdd(a.grad2d + 9 * (size_t)s_id[j + ei] + comp, g);
+    }
+  }
 }
 
 // Backward of list positions [start, end) of block blk (clipped to the block's walk), from the
 // forward's checkpoint `ck` when start > 0.
 __device__ __forceinline__ void bwd_chunk(const BwdArgs& a, int blk, int start, unsigned end,
-                                          const float4* ck, float2* s_uv, float4* s_co,
+                                          const float4* ck, float4* s_co, float4* s_m,
                                           float4* s_rgb, unsigned* s_id, float* s_red) {
   const Block bk = block_of(a.cam, blk);
   const int lane = threadIdx.x & 31;
   const uint2 rg = a.ranges[bk.tile];
   const int n = (rg.y > rg.x && !(*a.status & kStatusTimeout)) ? (int)(rg.y - rg.x) : 0;
-  const float fx0 = (float)bk.qx0 + 0.5f, fx1 = (float)bk.qx1 + 0.5f, fy = (float)bk.py + 0.5f;
+  const float2 fx = make_float2((float)bk.qx0 + 0.5f, (float)bk.qx1 + 0.5f);
+  const float fy = (float)bk.py + 0.5f;
   const float bx0 = (float)bk.px0 + 0.5f, by0 = (float)bk.py0 + 0.5f;
   PixB p0 = {}, p1 = {};
   p0.T = p1.T = 1.f;
@@ -571,7 +761,7 @@ __device__ __forceinline__ void bwd_chunk(const BwdArgs& a, int blk, int start, 
   const int span = (int)min((unsigned)__reduce_max_sync(0xffffffffu, max(p0.last, p1.last)), end);
   PixB2 pp;
   pp.T = make_float2(p0.T, p1.T);
-  pp.Gc = make_float2(p0.Gc, p1.Gc);
+  pp.nGc = make_float2(-p0.Gc, -p1.Gc);
   pp.Gr = make_float2(p0.Gr, p1.Gr);
   pp.Gg = make_float2(p0.Gg, p1.Gg);
   pp.Gb = make_float2(p0.Gb, p1.Gb);
@@ -580,57 +770,24 @@ __device__ __forceinline__ void bwd_chunk(const BwdArgs& a, int blk, int start, 
   int next = start;
   while (next < span) {
     __syncwarp();
-    const int cnt = stage_fill<true>(a.ids, rg.x, span, next, a.uv, a.co, a.rgb, bx0, by0,
-                                     a.op.alpha_min, s_uv, s_co, s_rgb, s_id);
-    // three entries per iteration, their 27 components summed over the warp at once (slots up
-    // to j + 2 <= kBatch + 1 exist; unused past cnt)
-    for (int j = 0; j < cnt; j += 3) {
-      float x[27];
-#pragma unroll
-      for (int k = 0; k < 27; ++k) x[k] = 0.f;
-      unsigned who[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const Entry e = load_entry(s_uv, s_co, s_rgb, j + i);
-        const unsigned pos = __float_as_uint(e.col.w);
-        const bool valid = j + i < cnt;
-        float dx0, dx1, dy, sg0, sg1;
-        sigma_pair(e.s, e.m, fx0, fx1, fy, dx0, dx1, dy, sg0, sg1);
-        bool c0, c1;
-        pixel_backward2(pp, e.s, e.col, sg0, sg1, dx0, dx1, dy, valid && pos < last0,
-                        valid && pos < last1, a.op, x + 9 * i, c0, c1);
-        who[i] = __ballot_sync(0xffffffffu, c0 || c1);
-      }
-      if ((who[0] | who[1] | who[2]) == 0) continue;
-      const float r = warp_sum27(x, s_red, lane);
-      const int ei = min(lane / 9, 2), comp = lane - 9 * ei;
-      // mean and conic gradients from the weighted moments of entry ei:
-      // d/du = -(ca Sx + cb Sy), d/dv = -(cb Sx + cc Sy), d/da = Sxx / 2, d/db = Sxy,
-      // d/dc = Syy / 2, with (ca, cb, cc) = ln 2 (2 a', b', 2 c') of the scaled conic
-      const float sx = __shfl_sync(0xffffffffu, r, 9 * ei);
-      const float sy = __shfl_sync(0xffffffffu, r, 9 * ei + 1);
-      const unsigned wi = ei == 0 ? who[0] : (ei == 1 ? who[1] : who[2]);
-      if (lane < 27 && wi != 0) {
-        float g = r;
-        if (comp <= 1) {
-          const float4 sc = s_co[j + ei];
-          const float ca = 2.f * kLn2 * sc.x, cb = kLn2 * sc.y, cc = 2.f * kLn2 * sc.z;
-          g = comp == 0 ? -(ca * sx + cb * sy) : -(cb * sx + cc * sy);
-        } else if (comp == 2 || comp == 4) {
-          g = 0.5f * r;
-        }
-        atomicAdd(a.grad2d + 9 * (size_t)s_id[j + ei] + comp, g);
-      }
-    }
+    bool clamp;
+    const int cnt = stage_fill(a.ids, rg.x, span, next, a.uv, a.co, a.rgb, bx0, by0, a.op, s_co,
+                               s_m, s_rgb, s_id, clamp);
+    if (!clamp) bwd_staged<false>(a, pp, fx, fy, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
+    else bwd_staged<true>(a, pp, fx, fy, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
   }
 }
 
-__global__ void __launch_bounds__(kSubThreads, 24) render_bwd_kernel(BwdArgs a) {
+// What bounds it: instruction issue (63M warp instructions at 1237x822 against 85M with scalar
+// selects on alpha and negated operands) and the shared-memory traffic of the per-entry sums.  20 CTAs
+// per SM leave 96 registers, so nothing spills: 79-95 us against 86-109 us at 24 CTAs and 82-98 us
+// at 16; 450 against 491 and 475 us for 2M Gaussians at 1920x1080 (530 us before).
+__global__ void __launch_bounds__(kSubThreads, 20) render_bwd_kernel(BwdArgs a) {
   pdl_prologue();
-  __shared__ float2 s_uv[kBatch + 2];
-  __shared__ float4 s_co[kBatch + 2];
-  __shared__ float4 s_rgb[kBatch + 2];
-  __shared__ unsigned s_id[kBatch + 2];
+  __shared__ float4 s_co[kGroup + 2];
+  __shared__ float4 s_m[kGroup + 2];
+  __shared__ float4 s_rgb[kGroup + 2];
+  __shared__ unsigned s_id[kGroup + 2];
   __shared__ __align__(16) float s_red[27 * kRedPitch];
   // the first n_item_ctas CTAs replay the listed chunks after the first of the long walks, the
   // others each a block's walk up to its first checkpoint
@@ -643,6 +800,7 @@ __global__ void __launch_bounds__(kSubThreads, 24) render_bwd_kernel(BwdArgs a) 
     const float4* ck = nullptr;
     if (item_cta) {
       const uint4 it = a.ck_items[i];
+      if (it.z == 0u) continue;                // a walk that ended before its checkpoint
       blk = (int)it.x; start = (int)it.y; end = it.z;
       ck = a.ckpt + (size_t)i * (kSub * kSub);
     } else {
@@ -650,7 +808,7 @@ __global__ void __launch_bounds__(kSubThreads, 24) render_bwd_kernel(BwdArgs a) 
       if (a.ckpt) end = a.ck_first[blk];
     }
     __syncwarp();
-    bwd_chunk(a, blk, start, end, ck, s_uv, s_co, s_rgb, s_id, s_red);
+    bwd_chunk(a, blk, start, end, ck, s_co, s_m, s_rgb, s_id, s_red);
     if (!item_cta) break;
   }
 }

@@ -310,6 +310,67 @@ def check_backward(ctx, case, r, bg, seed, state=None):
     return R
 
 
+# Walk lengths at the edges of the staging (64 positions), of the checkpoints (128) and of the
+# four (forward) and three (backward) entries per iteration; faint splats, so that no pixel ends
+# and every position counts, and opaque ones above alpha_max, some of which end pixels.
+@pytest.mark.parametrize("logit", [-2.5, 6.0])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 63, 64, 65, 127, 128, 129, 193, 261])
+def test_render_walk_lengths(ctx, n, logit):
+    s = sg.grid_scene((1, 1, 1), 5.0, n, 0, seed=500 + n)
+    s.gaussians.opacity_logits[:] = logit + 0.2 * s.gaussians.opacity_logits
+    s.gaussians.log_scales[:] += np.float32(np.log(2.0)) if logit < 0 else np.float32(0.0)
+    s.cameras = sg.ring_cameras(1, 9.0, np.zeros(3), 40, 24, seed=n, height_jitter=1.0)
+    case = Case(s, 0, fb=False)
+    r = run_forward(ctx, case, refresh=True)
+    R = oracle.render(case.sp, case.off, case.ids, case.cam.width, case.cam.height)
+    par.compare_render(r["out"].cpu().numpy(), r["state"].A_T.cpu().numpy()[..., 3], R, case.sp,
+                       case.off, case.ids, case.P, case.opt, case.cam)
+    got16 = r["refresh"].float().cpu().numpy()
+    assert np.abs(got16 - r["out"].cpu().numpy()).max() <= 2.0 ** -11      # fp16 rounding of [0, 1]
+    check_backward(ctx, case, r, None, seed=n)
+
+
+def test_render_indefinite_conic_is_walked(ctx):
+    """Projections given by the caller: a conic that is not positive definite (sigma falls below 0
+    away from the mean) and a NaN one are taken or skipped pixel by pixel, never culled by block,
+    in the forward and the backward."""
+    W = H = 32
+    n = 3
+    cam = ab.camera(sg.look_at((0.0, -5.0, 0.0), np.zeros(3), W, H))
+    proj = ab.Projected.alloc(n)
+    proj.uv.copy_(torch.tensor([[3.0, 4.0], [20.0, 18.0], [9.0, 9.0]]))
+    co = torch.tensor([[0.02, 0.05, 0.02, 0.5], [0.01, 0.0, 0.01, 0.6], [float("nan"), 0.0, 0.1, 0.7]])
+    proj.conic_opacity.copy_(co)
+    proj.rgb.copy_(torch.tensor([[1.0, 0.5, 0.25]] * n))
+    tiles = ab.Tiles.alloc(16, W, H)
+    tiles.ids[:12] = torch.tensor([0, 1, 2] * 4, dtype=torch.int32)
+    tiles.ranges.copy_(torch.tensor([[3 * t, 3 * t + 3] for t in range(4)], dtype=torch.int32))
+    out = torch.empty(H, W, 4, device="cuda")
+    st = ab.FwdState.alloc(W, H)
+    ab.abcd_render_composite_fwd(ctx, cam, None, proj, tiles, None, None, ab.ABCD_F16, None, out, st)
+    ctx.sync()
+    ys, xs = np.mgrid[0:H, 0:W] + 0.5
+    T = np.ones((H, W))
+    A = np.zeros((H, W))
+    edge = np.zeros((H, W), bool)
+    for k in range(2):
+        a, b, c, o = co[k].double().numpy()
+        dx, dy = xs - float(proj.uv[k, 0]), ys - float(proj.uv[k, 1])
+        sg_ = 0.5 * (a * dx * dx + c * dy * dy) + b * dx * dy
+        al = np.where((sg_ >= 0) & (o * np.exp(-sg_) >= 1 / 255), o * np.exp(-np.maximum(sg_, 0)), 0.0)
+        edge |= (np.abs(sg_) < 1e-4) | (np.abs(o * np.exp(-sg_) * 255 - 1) < 1e-3)
+        A += al * T
+        T *= 1 - al
+    got = out.cpu().numpy()
+    assert np.abs(got[..., 0] - A)[~edge].max() <= 1e-5
+    grad2d = torch.empty(n, 9, device="cuda")
+    ab.abcd_render_backward(ctx, cam, None, proj, tiles, None, None, ab.ABCD_F16, None, st,
+                            torch.ones(H, W, 3, device="cuda"), n, grad2d)
+    ctx.sync()
+    assert bool(torch.isfinite(grad2d).all())
+    assert bool((grad2d[2] == 0).all())
+
+
 @pytest.mark.parametrize("cam_idx", [0, 2])
 def test_render_backward_matches_oracle(ctx, tiny, cam_idx):
     case = Case(tiny, cam_idx, fb=True)
