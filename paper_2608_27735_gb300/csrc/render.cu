@@ -45,6 +45,7 @@ constexpr int kFwdUnroll = 4;                    // staged entries per iteration
 constexpr int kFwdRounds = 2;
 constexpr int kFwdGroup = kFwdRounds * kSubThreads;   // list positions the forward stages together
 constexpr int kCkChunk = 128;                    // list positions per backward chunk
+constexpr int kBwdUnroll = 5;                    // staged entries per iteration of the backward
 constexpr int kItemCtasPerSm = 16;               // backward CTAs that replay listed chunks
 static_assert(kCkChunk % kGroup == 0 && kCkChunk % kFwdGroup == 0,
               "checkpoints fall on staging group boundaries");
@@ -184,13 +185,12 @@ __device__ __forceinline__ int stage_fill(const unsigned* ids, unsigned start, i
     total += __popc(b);
   }
   next += kGroup;
-  // the loop over the survivors reads up to two slots past the last: a NaN sigma is taken by no
-  // pixel, and the rest must be finite (a zero weight times a non-finite value is not zero)
-  if (lane < 2) {
+  // the loop over the survivors reads past the last: a NaN sigma is taken by no pixel, and the
+  // rest must be finite (a zero weight times a non-finite value is not zero)
+  if (lane < kBwdUnroll - 1) {
     s_co[total + lane] = make_float4(__int_as_float(0x7fffffff), 0.f, 0.f, 0.f);
     s_m[total + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
     s_rgb[total + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-    s_id[total + lane] = 0u;
   }
   clamp = __any_sync(0xffffffffu, over);
   __syncwarp();
@@ -556,6 +556,7 @@ __global__ void __launch_bounds__(kSubThreads, 24) render_fwd_kernel(const __gri
   }
   if (bk.in0) store_pixel(a, (long long)bk.py * a.cam.width + bk.qx0, p0, bk.qx0, bk.py, bk.tile);
   if (bk.in1) store_pixel(a, (long long)bk.py * a.cam.width + bk.qx1, p1, bk.qx1, bk.py, bk.tile);
+  asm volatile("cp.async.wait_all;" ::: "memory");   // a walk that ended early has copies in flight
 }
 
 struct BwdArgs {
@@ -611,25 +612,27 @@ __device__ __forceinline__ void load_pixel_grad(const BwdArgs& a, long long p, i
 
 // Backward of the lane's two pixels for one list entry (selects, no branches): when the entry
 // contributed to a pixel (live: a position up to the pixel's last contributor; sigma within the
-// limit) gives in v the opacity and colour gradients (v[5..8]) and the moments of d = pixel - uv
-// weighted by dL/dsigma, (sum w dx, w dy, w dx^2, w dx dy, w dy^2) in v[0..4] (the conic and mean
-// gradients follow from them once per entry), and advances the replayed transmittance.  With
+// limit) adds up over the two pixels, into v: the opacity gradient, dL/dsigma dx, dL/dsigma dx^2
+// and the colour gradients, and advances the replayed transmittance.  (dL/dsigma is -opacity
+// times the opacity gradient's summand, and dy is the same along a row of the block, so these
+// six sums hold all nine gradients, see bwd_staged.)  With
 // G = dL/dA.rgb and G_a = dL/dA.a, the derivative of the loss w.r.t. an entry's alpha is
 //   T (G . col) - (K - G . C) / (1 - alpha),   K = G . A - G_a T_final,
 // C the colour accumulated up to and including the entry.  The two pixels' arithmetic is paired
 // through the packed two-lane fp32 instructions, which have no negated operands: the staged
-// opacity is negated, and so is the replayed G . C, so that none is needed.  The row offset dy is
-// factored out of the moment sums (sum t dy = (t0 + t1) dy).  The decisions (sigma, its limit)
-// are rounded exactly as the forward rounds them.  who0 / who1: whether the entry contributed to
-// each pixel.
+// opacity is negated, and so is the replayed G . C, so that none is needed.  The decisions
+// (sigma, its limit) are rounded exactly as the forward rounds them.  Returns whether the entry
+// contributed to either pixel.
+constexpr int kSums = 6;              // sums per entry
+
 struct PixB2 {
   float2 T, nGc, Gr, Gg, Gb, K;
 };
 
 template <bool CLAMP>
-__device__ __forceinline__ void pixel_backward2(PixB2& p, const Entry& e, float2 sg, float2 dx,
-                                                float dy, bool live0, bool live1, const Opts& op,
-                                                float* v, bool& who0, bool& who1) {
+__device__ __forceinline__ bool pixel_backward2(PixB2& p, const Entry& e, float2 sg, float2 dx,
+                                                bool live0, bool live1, const Opts& op,
+                                                float (&v)[kSums]) {
   const bool ok0 = live0 && takes(sg.x, e.m.z);
   const bool ok1 = live1 && takes(sg.y, e.m.z);
   // an entry that is not taken gets a sigma whose exponential is 0, and with it alpha and every
@@ -650,88 +653,79 @@ __device__ __forceinline__ void pixel_backward2(PixB2& p, const Entry& e, float2
   // d alpha / d opacity = G, d alpha / d sigma = -alpha; none of either where alpha was clamped
   if (CLAMP) da = make_float2(nraw.x >= -op.alpha_max ? da.x : 0.f, nraw.y >= -op.alpha_max ? da.y : 0.f);
   const float2 dg = __fmul2_rn(da, G);
-  const float2 ds = __fmul2_rn(da, nraw);
-  v[5] = dg.x + dg.y;
-  v[6] = fmaf(p.Gr.x, -nw.x, p.Gr.y * -nw.y);
-  v[7] = fmaf(p.Gg.x, -nw.x, p.Gg.y * -nw.y);
-  v[8] = fmaf(p.Gb.x, -nw.x, p.Gb.y * -nw.y);
-  const float2 t = __fmul2_rn(ds, dx);
-  const float ts = t.x + t.y, us = (ds.x + ds.y) * dy;
-  v[0] = ts;
-  v[1] = us;
+  const float2 t = __fmul2_rn(__fmul2_rn(da, nraw), dx);             // dL/dsigma dx
+  v[0] = dg.x + dg.y;
+  v[1] = t.x + t.y;
   v[2] = fmaf(t.x, dx.x, t.y * dx.y);
-  v[3] = ts * dy;
-  v[4] = us * dy;
+  v[3] = fmaf(p.Gr.x, -nw.x, p.Gr.y * -nw.y);
+  v[4] = fmaf(p.Gg.x, -nw.x, p.Gg.y * -nw.y);
+  v[5] = fmaf(p.Gb.x, -nw.x, p.Gb.y * -nw.y);
   p.T = __ffma2_rn(na, p.T, p.T);
-  who0 = ok0;
-  who1 = ok1;
+  return ok0 || ok1;
 }
 
-// Warp sum of 27 per-lane values through shared memory: each lane writes its row, lane l < 27
-// reads column l (32 values, 8 float4 loads; pitch 36 keeps stores and loads conflict-free)
-// and returns its sum (lanes past 26: column 26's).
+// Backward of the staged entries [0, cnt) at the lane's two pixels, kBwdUnroll entries per
+// iteration (past cnt a NaN sigma is taken by no pixel).  Each lane writes an entry's six sums to shared memory as row 6 i + k (pitch 36: no
+// bank conflicts in either direction); lane l then reads row l, whose float4 q holds the four
+// lanes of pixel row q, and takes the row's sum S = sum s_q and its moments S1 = sum s_q dy_q and
+// S2 = sum s_q dy_q^2 over the rows.  With (ca, cb, cc) = ln 2 (2 a', b', 2 c') of the scaled
+// conic, D = dL/dsigma = -o (the opacity gradient's summands):
+//   d/du = -(ca sum D dx + cb sum D dy),  d/dv = -(cb sum D dx + cc sum D dy),
+//   d/da = sum D dx^2 / 2,  d/db = sum D dx dy,  d/dc = sum D dy^2 / 2.
 constexpr int kRedPitch = 36;
+static_assert(kBwdUnroll * kSums <= 32, "one row per lane");
 
-__device__ __forceinline__ float warp_sum27(const float (&x)[27], float* red, int lane) {
-#pragma unroll
-  for (int k = 0; k < 27; ++k) red[k * kRedPitch + lane] = x[k];
-  __syncwarp();
-  const float4* col = reinterpret_cast<const float4*>(red + min(lane, 26) * kRedPitch);
-  float2 r0 = make_float2(0.f, 0.f), r1 = r0;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const float4 a = col[q];
-    r0 = __fadd2_rn(r0, make_float2(a.x, a.y));
-    r1 = __fadd2_rn(r1, make_float2(a.z, a.w));
-  }
-  __syncwarp();
-  r0 = __fadd2_rn(r0, r1);
-  return r0.x + r0.y;
-}
-
-// Backward of the staged entries [0, cnt) at the lane's two pixels, three entries per iteration,
-// their 27 components summed over the warp at once (slots up to cnt + 1 exist; past cnt a NaN
-// sigma is taken by no pixel).
 template <bool CLAMP>
 __device__ __forceinline__ void bwd_staged(const BwdArgs& a, PixB2& pp, float2 fx, float fy,
-                                           unsigned last0, unsigned last1, int cnt,
+                                           float by0, unsigned last0, unsigned last1, int cnt,
                                            const float4* s_co, const float4* s_m,
                                            const float4* s_rgb, const unsigned* s_id,
                                            float* s_red) {
   const int lane = threadIdx.x & 31;
-  for (int j = 0; j < cnt; j += 3) {
-    float x[27];
-    unsigned who[3];
+  const int ei = min(lane / kSums, kBwdUnroll - 1), comp = lane - kSums * ei;
+  for (int j = 0; j < cnt; j += kBwdUnroll) {
+    unsigned who = 0u;                               // bit i: entry j + i counts for some pixel
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < kBwdUnroll; ++i) {
       const Entry e = load_entry(s_co, s_m, s_rgb, j + i);
       const unsigned nxt = __float_as_uint(e.m.w);
       float2 dx, sg;
-      float dy;
+      float dy, v[kSums];
       sigma_pair(e.s, e.m, fx, fy, dx, dy, sg);
-      bool c0, c1;
-      pixel_backward2<CLAMP>(pp, e, sg, dx, dy, nxt <= last0, nxt <= last1, a.op, x + 9 * i, c0, c1);
-      who[i] = __ballot_sync(0xffffffffu, c0 || c1);
+      const bool c = pixel_backward2<CLAMP>(pp, e, sg, dx, nxt <= last0, nxt <= last1, a.op, v);
+      if (__any_sync(0xffffffffu, c)) who |= 1u << i;
+#pragma unroll
+      for (int k = 0; k < kSums; ++k) s_red[(kSums * i + k) * kRedPitch + lane] = v[k];
     }
-    if ((who[0] | who[1] | who[2]) == 0) continue;
-    const float r = warp_sum27(x, s_red, lane);
-    const int ei = min(lane / 9, 2), comp = lane - 9 * ei;
-    // mean and conic gradients from the weighted moments of entry ei:
-    // d/du = -(ca Sx + cb Sy), d/dv = -(cb Sx + cc Sy), d/da = Sxx / 2, d/db = Sxy,
-    // d/dc = Syy / 2, with (ca, cb, cc) = ln 2 (2 a', b', 2 c') of the scaled conic
-    const float sx = __shfl_sync(0xffffffffu, r, 9 * ei);
-    const float sy = __shfl_sync(0xffffffffu, r, 9 * ei + 1);
-    const unsigned wi = ei == 0 ? who[0] : (ei == 1 ? who[1] : who[2]);
-    if (lane < 27 && wi != 0) {
-      float g = r;
-      if (comp <= 1) {
-        const float4 sc = s_co[j + ei];
-        const float ca = 2.f * kLn2 * sc.x, cb = kLn2 * sc.y, cc = 2.f * kLn2 * sc.z;
-        g = comp == 0 ? -(ca * sx + cb * sy) : -(cb * sx + cc * sy);
-      } else if (comp == 2 || comp == 4) {
-        g = 0.5f * r;
+    if (who == 0u) continue;
+    __syncwarp();
+    const float4 sc = s_co[j + ei];    // a', b', c', -o
+    const float dy0 = by0 + s_m[j + ei].y;
+    const float4* row = reinterpret_cast<const float4*>(s_red + min(lane, kSums * kBwdUnroll - 1) * kRedPitch);
+    float S = 0.f, S1 = 0.f, S2 = 0.f;
+#pragma unroll
+    for (int q = 0; q < kSub; ++q) {
+      const float4 r = row[q];
+      const float2 h = __fadd2_rn(make_float2(r.x, r.y), make_float2(r.z, r.w));
+      const float sq = h.x + h.y, dyq = dy0 + (float)q, sd = sq * dyq;
+      S += sq;
+      S1 += sd;
+      S2 = fmaf(sd, dyq, S2);
+    }
+    __syncwarp();
+    const float sx = __shfl_sync(0xffffffffu, S, kSums * ei + 1);             // sum D dx
+    const float sy = sc.w * __shfl_sync(0xffffffffu, S1, kSums * ei);         // sum D dy
+    if (lane < kSums * kBwdUnroll && ((who >> ei) & 1u)) {
+      const float ca = 2.f * kLn2 * sc.x, cb = kLn2 * sc.y, cc = 2.f * kLn2 * sc.z;
+      float* g = a.grad2d + 9 * (size_t)s_id[j + ei];
+      const float g0 = comp == 1 ? -(ca * sx + cb * sy) : (comp == 2 ? 0.5f * S : S);
+      const int c0 = comp == 0 ? 5 : (comp == 1 ? 0 : (comp == 2 ? 2 : comp + 3));
+      atomicAdd(g + c0, g0);                         // o, u, a, r, g, b
+      if (comp < 3) {
+        const float g1 = comp == 0 ? 0.5f * sc.w * S2 : (comp == 1 ? S1 : -(cb * sx + cc * sy));
+        const int c1 = comp == 0 ? 4 : (comp == 1 ? 3 : 1);
+        atomicAdd(g + c1, g1);                       // c, b, v
       }
-      atomicAdd(a.grad2d + 9 * (size_t)s_id[j + ei] + comp, g);
     }
   }
 }
@@ -773,22 +767,24 @@ __device__ __forceinline__ void bwd_chunk(const BwdArgs& a, int blk, int start, 
     bool clamp;
     const int cnt = stage_fill(a.ids, rg.x, span, next, a.uv, a.co, a.rgb, bx0, by0, a.op, s_co,
                                s_m, s_rgb, s_id, clamp);
-    if (!clamp) bwd_staged<false>(a, pp, fx, fy, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
-    else bwd_staged<true>(a, pp, fx, fy, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
+    if (!clamp) bwd_staged<false>(a, pp, fx, fy, by0, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
+    else bwd_staged<true>(a, pp, fx, fy, by0, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
   }
 }
 
-// What bounds it: instruction issue (63M warp instructions at 1237x822 against 85M with scalar
-// selects on alpha and negated operands) and the shared-memory traffic of the per-entry sums.  20 CTAs
-// per SM leave 96 registers, so nothing spills: 79-95 us against 86-109 us at 24 CTAs and 82-98 us
-// at 16; 450 against 491 and 475 us for 2M Gaussians at 1920x1080 (530 us before).
+// What bounds it: shared memory and the gathers (the L1's data stage 65% busy at 1237x822, 84% for
+// dense tiles before the sums went by rows) and instruction issue (55%).  With nine sums per entry
+// in three entries per iteration: 95 and 79 us (two cameras, 100,000 Gaussians at 1237x822) and
+// 450 us (2M at 1920x1080); with six sums in five entries 87, 72 and 406 us; four entries 90, 75
+// and 427 us; staging through asynchronous copies 100, 80 and 467 us (more shared-memory traffic).
+// 20 CTAs per SM leave 96 registers, so nothing spills; 16 CTAs 94, 76 and 434 us.
 __global__ void __launch_bounds__(kSubThreads, 20) render_bwd_kernel(BwdArgs a) {
   pdl_prologue();
-  __shared__ float4 s_co[kGroup + 2];
-  __shared__ float4 s_m[kGroup + 2];
-  __shared__ float4 s_rgb[kGroup + 2];
-  __shared__ unsigned s_id[kGroup + 2];
-  __shared__ __align__(16) float s_red[27 * kRedPitch];
+  __shared__ float4 s_co[kGroup + kBwdUnroll - 1];
+  __shared__ float4 s_m[kGroup + kBwdUnroll - 1];
+  __shared__ float4 s_rgb[kGroup + kBwdUnroll - 1];
+  __shared__ unsigned s_id[kGroup];
+  __shared__ __align__(16) float s_red[kSums * kBwdUnroll * kRedPitch];
   // the first n_item_ctas CTAs replay the listed chunks after the first of the long walks, the
   // others each a block's walk up to its first checkpoint
   const int b = (int)blockIdx.x;

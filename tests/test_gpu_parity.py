@@ -311,7 +311,7 @@ def check_backward(ctx, case, r, bg, seed, state=None):
 
 
 # Walk lengths at the edges of the staging (64 positions), of the checkpoints (128) and of the
-# four (forward) and three (backward) entries per iteration; faint splats, so that no pixel ends
+# four (forward) and five (backward) entries per iteration; faint splats, so that no pixel ends
 # and every position counts, and opaque ones above alpha_max, some of which end pixels.
 @pytest.mark.parametrize("logit", [-2.5, 6.0])
 @pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 63, 64, 65, 127, 128, 129, 193, 261])
