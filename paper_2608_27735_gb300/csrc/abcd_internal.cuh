@@ -107,20 +107,6 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// Mask of the lanes whose value equals this lane's, for values 0..256 (256 marks an unused
-// lane; it matches only other unused lanes).  Nine ballots: the cost does not depend on how
-// many distinct values the warp holds, unlike __match_any_sync's.
-__device__ __forceinline__ unsigned match_byte(unsigned d) {
-  unsigned peers = 0xffffffffu;
-#pragma unroll
-  for (int b = 0; b < 9; ++b) {
-    const unsigned bit = (d >> b) & 1u;
-    const unsigned m = __ballot_sync(0xffffffffu, bit);
-    peers &= bit ? m : ~m;
-  }
-  return peers;
-}
-
 // Tiles the workspace orders for images of up to max_pixels pixels with sides up to 16384.
 inline long long max_order_tiles(long long max_pixels) { return max_pixels / 256 + 2048; }
 

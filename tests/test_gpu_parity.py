@@ -942,6 +942,37 @@ def test_bin_sort_wait_timeout_reported(ctx):
     assert torch.equal(tiles.ids[:K], ref_ids) and torch.equal(tiles.ranges, ref_rng)
 
 
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 64, 2000, 2432, 2433, 3071, 3072, 3073])
+@pytest.mark.parametrize("depths", ["random", "ties", "culled"])
+def test_small_blocks_order_as_the_radix_sort(ctx, n, depths):
+    """Blocks of up to 3072 Gaussians get their depth order by counting; their lists equal those
+    of the radix passes (which the look-back hook selects; the withheld tile does not exist)."""
+    W, H = 200, 120
+    g = torch.Generator(device="cuda").manual_seed(n)
+    proj = ab.Projected.alloc(n)
+    proj.uv.copy_(torch.rand(n, 2, generator=g, device="cuda") * torch.tensor([W + 40.0, H + 40.0], device="cuda") - 20.0)
+    s = 0.02 + 0.3 * torch.rand(n, generator=g, device="cuda")
+    proj.conic_opacity.copy_(torch.stack([s, 0.3 * s, s, 0.05 + 0.9 * torch.rand(n, generator=g, device="cuda")], 1))
+    proj.rgb.fill_(0.5)
+    z = 0.2 + 50.0 * torch.rand(n, generator=g, device="cuda")
+    proj.depth.copy_(torch.round(z / 10.0) * 10.0 + 0.5 if depths == "ties" else z)
+    proj.radius.fill_(30)
+    if depths == "culled":
+        proj.radius[torch.rand(n, generator=g, device="cuda") < 0.7] = 0
+    cam = ab.camera(sg.look_at((0.0, -5.0, 0.0), np.zeros(3), W, H))
+    got = []
+    for hook in (-1, 1 << 40):
+        tiles = ab.Tiles.alloc(1_000_000, W, H)
+        assert ab.lib().abcd_test_withhold_lookback(ctx.h, hook) == ab.ABCD_OK
+        ab.abcd_bin_sort(ctx, proj, n, cam, tiles)
+        ctx.sync()
+        K = int(tiles.count.item())
+        got.append((K, tiles.ids[:K].clone(), tiles.ranges.clone()))
+    assert got[0][0] == got[1][0] and torch.equal(got[0][2], got[1][2])
+    assert torch.equal(got[0][1], got[1][1])
+    assert n < 64 or got[0][0] > 0
+
+
 def test_invalid_arguments_rejected(ctx):
     cam = ab.abcd_camera()
     cam.width = 0
