@@ -37,7 +37,7 @@ struct Cam {               // camera as the kernels read it (by value)
 
 struct Opts {
   float near_z, dilation, alpha_max, alpha_min, t_min, guard;
-  float log2_alpha_min;    // -inf when alpha_min <= 0: no entry is too faint
+  float inv_alpha_min;     // 1 / alpha_min; inf when alpha_min <= 0: no entry is too faint
 };
 
 struct SHConst { float k[16]; };    // normalisation factors of the real SH basis

@@ -90,7 +90,7 @@ Opts make_opts(const abcd_render_opts* o) {
   r.alpha_max = o ? o->alpha_max : 0.99f;
   r.alpha_min = o ? o->alpha_min : 1.0f / 255.0f;
   r.t_min = o ? o->t_min : 1e-4f;
-  r.log2_alpha_min = r.alpha_min > 0.f ? (float)std::log2((double)r.alpha_min) : -INFINITY;
+  r.inv_alpha_min = r.alpha_min > 0.f ? 1.f / r.alpha_min : INFINITY;
   return r;
 }
 

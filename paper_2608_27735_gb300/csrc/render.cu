@@ -97,13 +97,21 @@ __device__ __forceinline__ float box_min_sigma2(float4 s, float X0, float Y0) {
   return fminf(q0, q1);
 }
 
-// Largest sigma * log2(e) at which an entry of opacity o still has alpha >= alpha_min,
-// log2(o / alpha_min), or -1 for an entry that never does.  A pixel takes the entry iff
-// 0 <= sigma' <= the limit, one unsigned comparison of the two values' bits (a negative or NaN
-// sigma' is above every limit).  lg2.approx is within 2^-22 of the logarithm, as ex2.approx is of
-// the exponential that the alpha itself comes from.
+// Largest sigma * log2(e) at which an entry of opacity o still has alpha >= alpha_min, or -1 for
+// an entry that never does.  A pixel takes the entry iff 0 <= sigma' <= the limit, one unsigned
+// comparison of the two values' bits (a negative or NaN sigma' is above every limit).  The limit
+// is the last float near log2(o / alpha_min) at which the alpha itself, o ex2.approx(-sigma'),
+// passes: lg2.approx alone is up to two units off, and pixels near the threshold would be decided
+// less exactly than by their alpha.
 __device__ __forceinline__ float sigma_limit(float o, const Opts& op) {
-  const float lim = fmaxf(__log2f(o) - op.log2_alpha_min, 0.f);
+  const float l = fmaxf(__log2f(o * op.inv_alpha_min), 0.f);
+  const int bits = max(__float_as_int(l), 2);
+  float lim = __int_as_float(bits - 2);
+#pragma unroll
+  for (int k = -1; k <= 2; ++k) {
+    const float c = __int_as_float(bits + k);
+    if (__fmul_rn(o, ex2_approx(-c)) >= op.alpha_min) lim = c;
+  }
   return ((o >= op.alpha_min) & (op.alpha_max >= op.alpha_min)) ? lim : -1.f;
 }
 
@@ -292,7 +300,7 @@ __device__ __forceinline__ Entry load_entry(const float4* s_co, const float4* s_
 
 // Front-to-back step of the lane's two pixels over U staged entries.  The alphas come first
 // (negated, 0 where an entry is not taken), then the transmittances after each entry, linked by
-// one FMA per entry; when no pixel of the warp falls below t_min among them (a vote), the
+// one multiplication per entry; when no pixel of the warp falls below t_min among them (a vote), the
 // colours are added without another test.  Otherwise the entries are taken one by one: the entry
 // that takes a pixel below t_min ends it and does not contribute.  CLAMP: some staged opacity
 // exceeds alpha_max (else o 2^-sigma' cannot).
@@ -317,7 +325,7 @@ __device__ __forceinline__ void blend(PixF2& p, const float4* s_co, const float4
 #pragma unroll
   for (int k = 0; k < U; ++k) {
     Tb[k] = T;
-    T = __ffma2_rn(na[k], T, T);
+    T = __fmul2_rn(T, __fadd2_rn(make_float2(1.f, 1.f), na[k]));
   }
   if (!__any_sync(0xffffffffu, fminf(T.x, T.y) < op.t_min)) {
     p.T = T;
@@ -338,7 +346,7 @@ __device__ __forceinline__ void blend(PixF2& p, const float4* s_co, const float4
   for (int k = 0; k < U; ++k) {
     const float4 col = s_rgb[k];
     const unsigned pos = __float_as_uint(s_m[k].w);
-    const float2 Tn = __ffma2_rn(na[k], p.T, p.T);
+    const float2 Tn = __fmul2_rn(p.T, __fadd2_rn(make_float2(1.f, 1.f), na[k]));
     const bool t0 = on0 && na[k].x < 0.f, t1 = on1 && na[k].y < 0.f;
     const bool u0 = t0 && !(Tn.x < op.t_min), u1 = t1 && !(Tn.y < op.t_min);
     on0 = on0 && (u0 || !t0);
@@ -432,7 +440,7 @@ __device__ __forceinline__ void fetch_group(const FwdArgs& a, const unsigned (&g
 // instructions and latency: the entries of the next 64 list positions are copied to shared
 // memory, and the ids of the 64 after them loaded, while the current ones are blended; the block
 // cull takes both lanes' rounds side by side without branches; four entries are evaluated
-// together whose states are linked by one FMA, with the end-of-pixel test voted on once per
+// together whose states are linked by one multiplication, with the end-of-pixel test voted on once per
 // four.  Against two entries at a time with their selects and 64 entries loaded when needed:
 // 33 -> 23 us (2,000 Gaussians, 128x128), 84 -> 62 us (100,000, 1237x822), 218 -> 189 us (2M,
 // 1920x1080); the refresh at 1237x822 77-98 -> 53-68 us.  Eight entries per iteration need 120
@@ -660,7 +668,7 @@ __device__ __forceinline__ bool pixel_backward2(PixB2& p, const Entry& e, float2
   v[3] = fmaf(p.Gr.x, -nw.x, p.Gr.y * -nw.y);
   v[4] = fmaf(p.Gg.x, -nw.x, p.Gg.y * -nw.y);
   v[5] = fmaf(p.Gb.x, -nw.x, p.Gb.y * -nw.y);
-  p.T = __ffma2_rn(na, p.T, p.T);
+  p.T = __fmul2_rn(p.T, oma);
   return ok0 || ok1;
 }
 
