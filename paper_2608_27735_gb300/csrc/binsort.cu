@@ -71,14 +71,12 @@ __device__ __forceinline__ int4 tile_rect(float2 m, int r, int tiles_x, int tile
 
 // Depth sort item of Gaussian i, bits(depth) << 32 | id (the key all ones when it is culled); q
 // receives the tile rectangle of its square (empty when culled).
-__device__ __forceinline__ u64 depth_item(const float* depth, const int* radius, const float2* uv,
-                                          int i, int tiles_x, int tiles_y, int4& q) {
-  const int r = radius[i];
-  q = make_int4(0, 0, 0, 0);
-  if (r > 0) q = tile_rect(uv[i], r, tiles_x, tiles_y);
+__device__ __forceinline__ u64 depth_item(float2 m, int r, float z, int i, int tiles_x,
+                                          int tiles_y, int4& q) {
+  q = tile_rect(m, r, tiles_x, tiles_y);
   const bool vis = r > 0 && q.x < q.z && q.y < q.w;
   if (!vis) q = make_int4(0, 0, 0, 0);
-  return ((u64)(vis ? __float_as_uint(depth[i]) : 0xFFFFFFFFu) << 32) | (unsigned)i;
+  return ((u64)(vis ? __float_as_uint(z) : 0xFFFFFFFFu) << 32) | (unsigned)i;
 }
 
 // Zeroes the words the binning adds to: per-row run counts and the tile rows' difference array
@@ -93,12 +91,12 @@ __device__ __forceinline__ void clear_rows(unsigned* rows_zero, int rows_words, 
 }
 
 // ---- depth order of a small block by counting: item i goes to the number of items smaller than
-// it.  n^2 comparisons, but one launch where the digit counts and four radix passes are five: with
-// 2,000 Gaussians abcd_bin_sort takes 38 us instead of 52.  Every CTA holds all items in shared
-// memory and places `per` of them, 256 / per threads each.  Also the tile rectangles.  Up to
-// kRankMax items, where the comparisons overtake the passes: abcd_bin_sort 36 against 50 us with
-// 1,000 Gaussians, 41 against 53 with 2,000, 59 against 56 with 4,000.
-constexpr int kRankMax = 3072;
+// it.  n^2 comparisons, but one launch where the digit counts and four radix passes are five.
+// Every CTA holds all keys in shared memory and places `per` items, 256 / per threads each.  Also
+// the tile rectangles.  Up to kRankMax items, where the comparisons overtake the passes:
+// abcd_bin_sort 35 against 50 us with 1,000 Gaussians, 38 against 53 with 2,000, 50 against 57
+// with 4,000, 57 against 61 with 6,000, 80 against 62 with 8,192.
+constexpr int kRankMax = 6144;
 constexpr int kRankThreads = 256;
 
 __global__ void __launch_bounds__(kRankThreads)
@@ -106,23 +104,61 @@ rank_sort_kernel(const float* depth, const int* radius, const float2* uv, int n,
                  int tiles_x, int tiles_y, u64* sorted, int4* rects, unsigned* rows_zero,
                  int rows_words, int* diff_zero, int diff_cells) {
   pdl_prologue();
-  extern __shared__ u64 s_item[];
+  extern __shared__ __align__(16) unsigned s_key[];  // [n rounded up to 4], all ones past n
   clear_rows(rows_zero, rows_words, diff_zero, diff_cells);
-  const int first = blockIdx.x * per;
-  for (int i = threadIdx.x; i < n; i += kRankThreads) {
-    int4 q;
-    s_item[i] = depth_item(depth, radius, uv, i, tiles_x, tiles_y, q);
-    if (i >= first && i < first + per) rects[i] = q;
+  const int first = blockIdx.x * per, quads = (n + 3) / 4;
+  constexpr int kBatch = 8;                          // items a thread has in flight
+  for (int b0 = 0; b0 < 4 * quads; b0 += kBatch * kRankThreads) {
+    float2 m[kBatch];
+    int rad[kBatch];
+    float z[kBatch];
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) {
+      const int i = b0 + k * kRankThreads + (int)threadIdx.x;
+      m[k] = i < n ? uv[i] : make_float2(0.f, 0.f);
+      rad[k] = i < n ? radius[i] : 0;
+      z[k] = i < n ? depth[i] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) {
+      const int i = b0 + k * kRankThreads + (int)threadIdx.x;
+      int4 q;
+      const unsigned key = (unsigned)(depth_item(m[k], rad[k], z[k], i, tiles_x, tiles_y, q) >> 32);
+      if (i < n && i >= first && i < first + per) rects[i] = q;
+      if (i < 4 * quads) s_key[i] = key;             // (radius 0 past n: all ones)
+    }
   }
   __syncthreads();
+  // thread `part` of item i takes every parts-th group of four keys: those before i count when
+  // they are at most the item's (equal keys: the smaller id comes first), those behind it when
+  // they are smaller
   const int parts = kRankThreads / per;              // 4 to 16 threads, in one warp
-  const int i = first + (int)threadIdx.x / parts, part = threadIdx.x % parts;
-  const u64 x = i < n ? s_item[i] : 0ull;
+  const int i = min(first + (int)threadIdx.x / parts, n - 1), part = threadIdx.x % parts;
+  const unsigned x = s_key[i];
+  const uint4* s4 = reinterpret_cast<const uint4*>(s_key);
+  const int own = i / 4, below = (own - part + parts - 1) / parts;   // groups of this thread before i's
+  const int all = (quads - part + parts - 1) / parts;
   int r = 0;
-#pragma unroll 8
-  for (int j = part; j < n; j += parts) r += s_item[j] < x;
+#pragma unroll 4
+  for (int k = 0; k < below; ++k) {
+    const uint4 v = s4[k * parts + part];
+    r += (v.x <= x) + (v.y <= x) + (v.z <= x) + (v.w <= x);
+  }
+  const bool mine = own % parts == part;
+  if (mine) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const unsigned v = s_key[4 * own + e];
+      r += v < x || (v == x && 4 * own + e < i);
+    }
+  }
+#pragma unroll 4
+  for (int k = below + (mine ? 1 : 0); k < all; ++k) {
+    const uint4 v = s4[k * parts + part];
+    r += (v.x < x) + (v.y < x) + (v.z < x) + (v.w < x);
+  }
   for (int o = parts >> 1; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  if (part == 0 && i < n) sorted[r] = x;
+  if (part == 0 && first + (int)threadIdx.x / parts < n) sorted[r] = ((u64)x << 32) | (unsigned)i;
 }
 
 // ---- per Gaussian: depth key (bits(depth) << 32 | id, all ones when culled) and the tile
@@ -144,7 +180,7 @@ __global__ void keys_rects_kernel(const float* depth, const int* radius, const f
   unsigned key = 0xFFFFFFFFu;
   if (i < n) {
     int4 q;
-    const u64 x = depth_item(depth, radius, uv, i, tiles_x, tiles_y, q);
+    const u64 x = depth_item(uv[i], radius[i], depth[i], i, tiles_x, tiles_y, q);
     rects[i] = q;
     items[i] = x;
     key = (unsigned)(x >> 32);
@@ -1384,9 +1420,7 @@ extern "C" abcd_status abcd_bin_sort(abcd_ctx* ctx, const abcd_projected* proj, 
   if (rank) {
     int per = 16;                                    // items per CTA: 64 at most, one CTA per SM
     while (per < 64 && (n + per - 1) / per > ctx->num_sms) per <<= 1;
-    const size_t smem = sizeof(u64) * (size_t)n;
-    e = ensure_smem(ctx, (const void*)rank_sort_kernel, smem);
-    if (e != cudaSuccess) return fail(ctx, ABCD_ERR_CUDA, "rank sort smem: %s", cudaGetErrorString(e));
+    const size_t smem = sizeof(uint4) * (size_t)((n + 3) / 4);
     by_depth = ctx->ws.dsort[0];
     if ((s = check_launch(ctx, "rank_sort_kernel",
                           launch_pdl(rank_sort_kernel, dim3((n + per - 1) / per), dim3(kRankThreads),

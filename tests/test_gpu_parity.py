@@ -942,10 +942,10 @@ def test_bin_sort_wait_timeout_reported(ctx):
     assert torch.equal(tiles.ids[:K], ref_ids) and torch.equal(tiles.ranges, ref_rng)
 
 
-@pytest.mark.parametrize("n", [1, 15, 16, 17, 64, 2000, 2432, 2433, 3071, 3072, 3073])
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 64, 2000, 2432, 2433, 4097, 6143, 6144, 6145])
 @pytest.mark.parametrize("depths", ["random", "ties", "culled"])
 def test_small_blocks_order_as_the_radix_sort(ctx, n, depths):
-    """Blocks of up to 3072 Gaussians get their depth order by counting; their lists equal those
+    """Blocks of up to 6144 Gaussians get their depth order by counting; their lists equal those
     of the radix passes (which the look-back hook selects; the withheld tile does not exist)."""
     W, H = 200, 120
     g = torch.Generator(device="cuda").manual_seed(n)
