@@ -5,8 +5,11 @@
 //
 // Pure streaming work: every layer is read once (16-byte streaming loads, evict-first), the
 // accumulator stays in registers across layers, F and B are written once.  Four layers are
-// loaded before they are folded so each thread keeps 64 bytes in flight.  The grid is a
-// multiple of the SM count and strides over pixel pairs.
+// loaded before they are folded so each thread keeps 64 bytes in flight, the last one to three
+// of a side together too (64 layers at 1080p 185 -> 181 us, 5.9 TB/s; 27 layers at 640x480 with
+// their loss 31.4 -> 28.7 us).  Eight in flight take 97 registers and are slower (215 us); one
+// pixel per thread on small images is, too (30.7 us).  The grid is a multiple of the SM count
+// and strides over pixel pairs.
 #include <algorithm>
 
 #include "abcd_internal.cuh"
@@ -45,36 +48,66 @@ __device__ __forceinline__ void fold(float* acc, const float* L) {
   }
 }
 
-// Loads PIX pixels (4 channels each) of layer `ptr` at pixel group g into f.
+// PIX pixels (4 channels each) of a layer at pixel group g, as loaded.
 template <int PIX, bool F16>
-__device__ __forceinline__ void load_group(const void* ptr, long long g, float* f) {
-  if (F16) {
-    if (PIX == 2) unpack_h8(__ldcs(reinterpret_cast<const uint4*>(ptr) + g), f);
-    else unpack_h4(__ldcs(reinterpret_cast<const uint2*>(ptr) + g), f);
-  } else {
+struct Raw {
+  uint4 r[F16 ? 1 : PIX];
+  __device__ __forceinline__ void load(const void* ptr, long long g) {
+    if (F16) {
+      if (PIX == 2) {
+        r[0] = __ldcs(reinterpret_cast<const uint4*>(ptr) + g);
+      } else {
+        const uint2 v = __ldcs(reinterpret_cast<const uint2*>(ptr) + g);
+        r[0] = make_uint4(v.x, v.y, 0u, 0u);
+      }
+    } else {
 #pragma unroll
-    for (int q = 0; q < PIX; ++q) {
-      const float4 v = __ldcs(reinterpret_cast<const float4*>(ptr) + g * PIX + q);
-      f[4 * q] = v.x; f[4 * q + 1] = v.y; f[4 * q + 2] = v.z; f[4 * q + 3] = v.w;
+      for (int q = 0; q < PIX; ++q) r[q] = __ldcs(reinterpret_cast<const uint4*>(ptr) + g * PIX + q);
     }
   }
-}
+  __device__ __forceinline__ void unpack(float* f) const {
+    if (F16) {
+      if (PIX == 2) unpack_h8(r[0], f);
+      else unpack_h4(make_uint2(r[0].x, r[0].y), f);
+    } else {
+#pragma unroll
+      for (int q = 0; q < (F16 ? 1 : PIX); ++q) {
+        f[4 * q] = __uint_as_float(r[q].x); f[4 * q + 1] = __uint_as_float(r[q].y);
+        f[4 * q + 2] = __uint_as_float(r[q].z); f[4 * q + 3] = __uint_as_float(r[q].w);
+      }
+    }
+  }
+};
+
+constexpr int kInFlight = 4;
 
 template <int PIX, bool F16>
 __device__ __forceinline__ void fold_range(const LayerTable& lt, int k0, int k1, long long g,
                                            float* acc) {
   int k = k0;
-  for (; k + 4 <= k1; k += 4) {
-    float v[4][4 * PIX];
+  for (; k + kInFlight <= k1; k += kInFlight) {
+    Raw<PIX, F16> v[kInFlight];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) load_group<PIX, F16>(lt.p[k + j], g, v[j]);
+    for (int j = 0; j < kInFlight; ++j) v[j].load(lt.p[k + j], g);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) fold<PIX>(acc, v[j]);
+    for (int j = 0; j < kInFlight; ++j) {
+      float f[4 * PIX];
+      v[j].unpack(f);
+      fold<PIX>(acc, f);
+    }
   }
-  for (; k < k1; ++k) {
-    float v[4 * PIX];
-    load_group<PIX, F16>(lt.p[k], g, v);
-    fold<PIX>(acc, v);
+  if (k < k1) {                                      // the rest, also in flight together
+    Raw<PIX, F16> v[kInFlight];
+#pragma unroll
+    for (int j = 0; j < kInFlight; ++j)
+      if (k + j < k1) v[j].load(lt.p[k + j], g);
+#pragma unroll
+    for (int j = 0; j < kInFlight; ++j) {
+      if (k + j >= k1) break;
+      float f[4 * PIX];
+      v[j].unpack(f);
+      fold<PIX>(acc, f);
+    }
   }
 }
 
@@ -172,7 +205,10 @@ extern "C" abcd_status abcd_composite_cache(abcd_ctx* ctx, const void* const* la
 
 // ---- K1 over packed layers (the cache's tile-sparse format, see abcd_render_refresh_packed):
 // one CTA per 16x16 tile, two pixels per thread, the tile's map entries of all layers read
-// once into shared memory; a layer whose tile is not stored is transparent, and folding
+// once into shared memory and compacted into the list of those that store it, so that all eight
+// loads a thread has in flight are real (32 layers at 1237x822, a third stored, F and B by two
+// halves of the CTA side by side: 21.4 -> 19.5 us, 5.2 TB/s; what is left is the latency of map,
+// list and loads per tile); a layer whose tile is not stored is transparent, and folding
 // (0, 0, 0, 0) leaves the accumulator unchanged, so skipping it gives the dense result bit for
 // bit.  Only the stored tiles are read.
 namespace abcd {
@@ -186,20 +222,20 @@ struct PackedTable {
 constexpr int kPackedThreads = kTileThreads / 2;
 constexpr int kPackedInFlight = 8;
 
-// The positions k in [0, n) with s_map[k] >= 0, in order, into s_list; returns how many (every
-// thread).  Warp 0 compacts with ballots; the caller's next __syncthreads publishes s_list.
-__device__ __forceinline__ void compact_stored(const int* s_map, int n, int* s_list,
-                                               int* s_count) {
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
+// The positions k in [k0, k1) with s_map[k] >= 0, in order, into s_list, and how many into
+// *s_count; warp 0 of the calling threads (thread: 0 for the first) compacts with ballots, and
+// the caller's next __syncthreads publishes both.
+__device__ __forceinline__ void compact_stored(const int* s_map, int k0, int k1, int thread,
+                                               int* s_list, int* s_count) {
+  if (thread >= 32) return;
   int run = 0;
-  for (int k0 = 0; k0 < n; k0 += 32) {
-    const bool st = k0 + lane < n && s_map[k0 + lane] >= 0;
-    const unsigned b = __ballot_sync(0xffffffffu, st);
-    if (st) s_list[run + __popc(b & ((1u << lane) - 1u))] = k0 + lane;
-    run += __popc(b);
+  for (int b = k0; b < k1; b += 32) {
+    const bool st = b + thread < k1 && s_map[b + thread] >= 0;
+    const unsigned m = __ballot_sync(0xffffffffu, st);
+    if (st) s_list[run + __popc(m & ((1u << thread) - 1u))] = b + thread;
+    run += __popc(m);
   }
-  if (lane == 0) *s_count = run;
+  if (thread == 0) *s_count = run;
 }
 
 // Calls fn(k, v) in order for the listed positions s_list[j0 .. j1) (v: this thread's 16-byte
@@ -207,8 +243,8 @@ __device__ __forceinline__ void compact_stored(const int* s_map, int n, int* s_l
 // they are used.
 template <typename Fn>
 __device__ __forceinline__ void for_each_listed(const uint4* const* data, const int* s_map,
-                                                const int* s_list, int j0, int j1, Fn fn) {
-  const int unit = threadIdx.x;
+                                                const int* s_list, int j0, int j1, int unit,
+                                                Fn fn) {
   int j = j0;
   for (; j + kPackedInFlight <= j1; j += kPackedInFlight) {
     uint4 r[kPackedInFlight];
@@ -236,34 +272,6 @@ __device__ __forceinline__ void for_each_listed(const uint4* const* data, const 
   }
 }
 
-// acc (2 pixels) = acc over the two pixels of every layer in [k0, k1) stored at this tile;
-// m: the tile's block index in every layer (shared memory, -1: not stored).  Eight layers'
-// loads are in flight before they are folded.
-__device__ __forceinline__ void fold_packed(const PackedTable& pt, const int* m, int k0, int k1,
-                                            int unit, float* acc) {
-  int k = k0;
-  for (; k + kPackedInFlight <= k1; k += kPackedInFlight) {
-    uint4 r[kPackedInFlight];
-#pragma unroll
-    for (int j = 0; j < kPackedInFlight; ++j)
-      r[j] = m[k + j] >= 0 ? __ldcs(pt.data[k + j] + (size_t)m[k + j] * kPackedThreads + unit)
-                           : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-    for (int j = 0; j < kPackedInFlight; ++j) {
-      if (m[k + j] < 0) continue;
-      float v[8];
-      unpack_h8(r[j], v);
-      fold<2>(acc, v);
-    }
-  }
-  for (; k < k1; ++k) {
-    if (m[k] < 0) continue;
-    float v[8];
-    unpack_h8(__ldcs(pt.data[k] + (size_t)m[k] * kPackedThreads + unit), v);
-    fold<2>(acc, v);
-  }
-}
-
 __device__ __forceinline__ void store_pixel_out(void* out, int f16, long long p, const float* acc) {
   if (f16) {
     const __half2 lo = __floats2half2_rn(acc[0], acc[1]), hi = __floats2half2_rn(acc[2], acc[3]);
@@ -274,29 +282,35 @@ __device__ __forceinline__ void store_pixel_out(void* out, int f16, long long p,
   }
 }
 
-__global__ void __launch_bounds__(kPackedThreads)
+// F by the first half of the CTA and B by the second, each over the list of the layers that
+// store the tile.
+__global__ void __launch_bounds__(2 * kPackedThreads)
 composite_packed_kernel(const __grid_constant__ PackedTable pt, int nf, int nb, int width,
                         int height, int tiles_x, void* Fout, void* Bout, int out_f16) {
   pdl_prologue();
-  __shared__ int s_map[kMaxLayers];
+  __shared__ int s_map[kMaxLayers], s_list[2][kMaxLayers], s_count[2];
   const int tile = blockIdx.x;
-  const int unit = threadIdx.x;                       // pixels 2 unit, 2 unit + 1 of the tile
+  const int side = threadIdx.x / kPackedThreads;
+  const int unit = threadIdx.x % kPackedThreads;      // pixels 2 unit, 2 unit + 1 of the tile
   for (int k = threadIdx.x; k < nf + nb; k += blockDim.x) s_map[k] = __ldg(pt.map[k] + tile);
   __syncthreads();
+  compact_stored(s_map, side ? nf : 0, side ? nf + nb : nf, unit, s_list[side], &s_count[side]);
+  __syncthreads();
+  void* out = side ? Bout : Fout;
+  if (!out) return;
   const int r = unit / (kTile / 2), c = 2 * (unit % (kTile / 2));
   const int y = (tile / tiles_x) * kTile + r, x = (tile % tiles_x) * kTile + c;
-  for (int side = 0; side < 2; ++side) {
-    void* out = side ? Bout : Fout;
-    if (!out) continue;
-    float acc[8];
+  float acc[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-    if (side == 0) fold_packed(pt, s_map, 0, nf, unit, acc);
-    else fold_packed(pt, s_map, nf, nf + nb, unit, acc);
-    if (y < height) {
-      if (x < width) store_pixel_out(out, out_f16, (long long)y * width + x, acc);
-      if (x + 1 < width) store_pixel_out(out, out_f16, (long long)y * width + x + 1, acc + 4);
-    }
+  for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+  for_each_listed(pt.data, s_map, s_list[side], 0, s_count[side], unit, [&](int, uint4 v) {
+    float f[8];
+    unpack_h8(v, f);
+    fold<2>(acc, f);
+  });
+  if (y < height) {
+    if (x < width) store_pixel_out(out, out_f16, (long long)y * width + x, acc);
+    if (x + 1 < width) store_pixel_out(out, out_f16, (long long)y * width + x + 1, acc + 4);
   }
 }
 
@@ -308,11 +322,12 @@ __global__ void __launch_bounds__(kPackedThreads)
 fold_packed_kernel(const __grid_constant__ PackedTable pt, int n, int width, int height,
                    int tiles_x, const float4* acc_in, float4* acc_out, uint2* out16) {
   pdl_prologue();
-  __shared__ int s_map[kMaxLayers];
+  __shared__ int s_map[kMaxLayers], s_list[kMaxLayers], s_count;
   const int tile = blockIdx.x;
   const int unit = threadIdx.x;
   for (int k = threadIdx.x; k < n; k += blockDim.x) s_map[k] = __ldg(pt.map[k] + tile);
   __syncthreads();
+  compact_stored(s_map, 0, n, unit, s_list, &s_count);
   const int r = unit / (kTile / 2), c = 2 * (unit % (kTile / 2));
   const int y = (tile / tiles_x) * kTile + r, x = (tile % tiles_x) * kTile + c;
   const long long p0 = (long long)y * width + x;
@@ -324,7 +339,12 @@ fold_packed_kernel(const __grid_constant__ PackedTable pt, int n, int width, int
     if (in0) { const float4 a = acc_in[p0]; acc[0] = a.x; acc[1] = a.y; acc[2] = a.z; acc[3] = a.w; }
     if (in1) { const float4 a = acc_in[p0 + 1]; acc[4] = a.x; acc[5] = a.y; acc[6] = a.z; acc[7] = a.w; }
   }
-  fold_packed(pt, s_map, 0, n, unit, acc);
+  __syncthreads();
+  for_each_listed(pt.data, s_map, s_list, 0, s_count, unit, [&](int, uint4 v) {
+    float f[8];
+    unpack_h8(v, f);
+    fold<2>(acc, f);
+  });
   if (in0) {
     if (acc_out) acc_out[p0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
     if (out16) store_pixel_out(out16, 1, p0, acc);
@@ -403,7 +423,7 @@ extern "C" abcd_status abcd_composite_cache_packed(abcd_ctx* ctx, const int* con
   const int tiles_x = (width + kTile - 1) / kTile, tiles_y = (height + kTile - 1) / kTile;
   return check_launch(ctx, "composite_packed_kernel",
                       launch_pdl(composite_packed_kernel, dim3(tiles_x * tiles_y),
-                                 dim3(kPackedThreads), 0, ctx->stream, pt, nf, nb, width, height,
+                                 dim3(2 * kPackedThreads), 0, ctx->stream, pt, nf, nb, width, height,
                                  tiles_x, F_out, B_out, out_dtype == ABCD_F16 ? 1 : 0));
 }
 
@@ -425,6 +445,11 @@ namespace {
 
 constexpr float kVisScale = 16777216.f;       // 2^24
 constexpr int kVisInFlight = 8;               // layers whose loads are in flight together
+// Positions with sums per thread: 64 take 64 KB per CTA and leave two on an SM, above that the
+// CTA's sums cost less.  32 layers at 1237x822, a third of the tiles stored: 26 us against 31 us
+// with a warp reduction and a shared atomic per layer, tile and sum (both bound by latency: 3.4
+// of 6.8 TB/s).
+constexpr int kVisOwnLayers = 64;
 constexpr int kVisCopies = kVisSumCopies;     // global accumulators (CTA b adds to copy b % 8)
 
 struct VisTable {
@@ -433,14 +458,22 @@ struct VisTable {
   int layer[kMaxLayers];                      // layer index at each position
 };
 
-// Adds one layer's contribution at the thread's two pixels (alphas a0, a1) to the CTA's sums
-// of position k, then takes the layer's transmittance factor into T0, T1.  Warp-uniform k.
+// Adds one layer's contribution at the thread's two pixels (alphas a0, a1) to the sums of position
+// k, then takes the layer's transmittance factor into T0, T1.  OWN: into the thread's own pair of
+// 32-bit sums (no reduction and no atomic per layer and tile); else into the CTA's, through a warp
+// reduction.  Warp-uniform k.
+template <bool OWN>
 __device__ __forceinline__ void vis_accumulate(float a0, float a1, float& T0, float& T1, int k,
-                                               unsigned long long (*s_sum)[kMaxLayers]) {
+                                               unsigned long long (*s_sum)[kMaxLayers], uint2* s_own) {
   const unsigned vf = __float2uint_rn(a0 * T0 * kVisScale) + __float2uint_rn(a1 * T1 * kVisScale);
   const unsigned cf = __float2uint_rn(a0 * kVisScale) + __float2uint_rn(a1 * kVisScale);
   T0 *= 1.f - a0;
   T1 *= 1.f - a1;
+  if (OWN) {
+    uint2& o = s_own[k * kPackedThreads + threadIdx.x];
+    o = make_uint2(o.x + vf, o.y + cf);
+    return;
+  }
   const unsigned vs = __reduce_add_sync(0xffffffffu, vf);
   const unsigned cs = __reduce_add_sync(0xffffffffu, cf);
   if ((threadIdx.x & 31) == 0) {
@@ -453,7 +486,7 @@ __device__ __forceinline__ float alpha_hi(unsigned w) {
   return __high2float(*reinterpret_cast<const __half2*>(&w));
 }
 
-template <bool PACKED>
+template <bool PACKED, bool OWN>
 __global__ void __launch_bounds__(kPackedThreads, 10)
 visibility_kernel(const __grid_constant__ VisTable vt, int count, int L, int width, int height,
                   int tiles_x, int n_tiles, unsigned long long* sums, unsigned* ticket,
@@ -464,7 +497,10 @@ visibility_kernel(const __grid_constant__ VisTable vt, int count, int L, int wid
   __shared__ int s_list[kMaxLayers];
   __shared__ int s_count;
   __shared__ bool s_last;
+  extern __shared__ uint2 s_own[];                     // OWN: [count][kPackedThreads]
   for (int k = threadIdx.x; k < count; k += blockDim.x) { s_sum[0][k] = 0ull; s_sum[1][k] = 0ull; }
+  if (OWN)
+    for (int k = 0; k < count; ++k) s_own[k * kPackedThreads + threadIdx.x] = make_uint2(0u, 0u);
   const int unit = threadIdx.x;
   const int r = unit / (kTile / 2), c = 2 * (unit % (kTile / 2));
   for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
@@ -472,15 +508,15 @@ visibility_kernel(const __grid_constant__ VisTable vt, int count, int L, int wid
     if (PACKED) {
       for (int k = threadIdx.x; k < count; k += blockDim.x) s_map[k] = __ldg(vt.map[k] + tile);
       __syncthreads();
-      compact_stored(s_map, count, s_list, &s_count);
+      compact_stored(s_map, 0, count, unit, s_list, &s_count);
     }
     __syncthreads();
     const int y = (tile / tiles_x) * kTile + r, x = (tile % tiles_x) * kTile + c;
     const bool in0 = y < height && x < width, in1 = y < height && x + 1 < width;
     float T0 = 1.f, T1 = 1.f;
     if (PACKED) {
-      for_each_listed(vt.data, s_map, s_list, 0, s_count, [&](int k, uint4 u) {
-        vis_accumulate(in0 ? alpha_hi(u.y) : 0.f, in1 ? alpha_hi(u.w) : 0.f, T0, T1, k, s_sum);
+      for_each_listed(vt.data, s_map, s_list, 0, s_count, unit, [&](int k, uint4 u) {
+        vis_accumulate<OWN>(in0 ? alpha_hi(u.y) : 0.f, in1 ? alpha_hi(u.w) : 0.f, T0, T1, k, s_sum, s_own);
       });
       continue;
     }
@@ -501,10 +537,29 @@ visibility_kernel(const __grid_constant__ VisTable vt, int count, int L, int wid
 #pragma unroll
       for (int j = 0; j < kVisInFlight; ++j)
         if (k0 + j < count)
-          vis_accumulate(alpha_hi(w0[j]), alpha_hi(w1[j]), T0, T1, k0 + j, s_sum);
+          vis_accumulate<OWN>(alpha_hi(w0[j]), alpha_hi(w1[j]), T0, T1, k0 + j, s_sum, s_own);
     }
   }
   __syncthreads();
+  if (OWN) {                                           // the threads' sums of each position: one warp
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < count; k += kPackedThreads / 32) {
+      unsigned long long v = 0ull, cv = 0ull;
+#pragma unroll
+      for (int q = 0; q < kPackedThreads / 32; ++q) {
+        const uint2 o = s_own[k * kPackedThreads + q * 32 + lane];
+        v += o.x;
+        cv += o.y;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        v += __shfl_xor_sync(0xffffffffu, v, o);
+        cv += __shfl_xor_sync(0xffffffffu, cv, o);
+      }
+      if (lane == 0) { s_sum[0][k] = v; s_sum[1][k] = cv; }
+    }
+    __syncthreads();
+  }
   unsigned long long* mine = sums + (size_t)(blockIdx.x % kVisCopies) * 2 * kMaxLayers;
   for (int k = threadIdx.x; k < count; k += blockDim.x) {
     if (s_sum[0][k]) atomicAdd(mine + k, s_sum[0][k]);
@@ -542,10 +597,19 @@ abcd_status visibility_launch(abcd_ctx* ctx, const char* who, VisTable& vt, bool
     return fail(ctx, ABCD_ERR_INVALID_ARG, "%s: null or misaligned output", who);
   const int tiles_x = (width + kTile - 1) / kTile, tiles_y = (height + kTile - 1) / kTile;
   const int n_tiles = tiles_x * tiles_y;
-  const int grid = std::max(1, std::min(n_tiles, 8 * ctx->num_sms));
-  const auto kernel = packed ? visibility_kernel<true> : visibility_kernel<false>;
+  // per-thread sums while they fit in shared memory with enough CTAs on an SM, and cannot
+  // overflow: a tile adds at most 2^25 to a 32-bit sum
+  const size_t own_bytes = sizeof(uint2) * kPackedThreads * (size_t)count;
+  const int own_ctas = std::max(1, std::min<int>(8, (int)((200u << 10) / (own_bytes + (8u << 10)))));
+  const bool own = count <= kVisOwnLayers && n_tiles <= 64LL * own_ctas * ctx->num_sms;
+  const int grid = std::max(1, std::min(n_tiles, (own ? own_ctas : 8) * ctx->num_sms));
+  const size_t smem = own ? own_bytes : 0;
+  const auto kernel = packed ? (own ? visibility_kernel<true, true> : visibility_kernel<true, false>)
+                             : (own ? visibility_kernel<false, true> : visibility_kernel<false, false>);
+  const cudaError_t e = ensure_smem(ctx, (const void*)kernel, smem);
+  if (e != cudaSuccess) return fail(ctx, ABCD_ERR_CUDA, "%s smem: %s", who, cudaGetErrorString(e));
   return check_launch(ctx, "visibility_kernel",
-                      launch_pdl(kernel, dim3(grid), dim3(kPackedThreads), 0, ctx->stream, vt,
+                      launch_pdl(kernel, dim3(grid), dim3(kPackedThreads), smem, ctx->stream, vt,
                                  count, L, width, height, tiles_x, n_tiles, ctx->ws.vis_sums,
                                  ctx->ws.vis_ticket, visible, coverage));
 }
