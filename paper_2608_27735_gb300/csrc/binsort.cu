@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(kOsThreads, 2)
 onesweep_kernel(const T* in, T* out, unsigned* out_ids, unsigned id_mask, long long n_static,
                 const long long* n_dev, long long cap, int shift, const unsigned* gh, u64* state,
                 unsigned* ctr, unsigned epoch, unsigned* status, unsigned spin_limit,
-                long long withhold, const unsigned* krange) {
+                long long withhold, const unsigned* krange, unsigned resident) {
   pdl_prologue();
   constexpr unsigned BINS = 1u << BITS, MASK = BINS - 1;
   constexpr int U = 64 / (int)sizeof(T);          // items per lane: 64 bytes in flight
@@ -568,11 +568,19 @@ onesweep_kernel(const T* in, T* out, unsigned* out_ids, unsigned id_mask, long l
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const KeyMap km = key_map(krange);
+  // Tiles that are all resident at once need no claims: CTA b takes tile b (and the tiles it
+  // waits for are running, or are started as soon as another kernel's CTA ends).  That saves
+  // three round trips per pass (the claim, the claim that finds nothing left, the counters'
+  // reset): a pass over 100,000 keys 12.0 -> 10.2 us, abcd_bin_sort 93 -> 82 us there.
+  const bool fixed = n_tiles <= (long long)resident;
+  if (fixed && blockIdx.x >= n_tiles) return;
   while (s_copy) {                                   // block-uniform (set before the scan's barriers)
-    if (threadIdx.x == 0) s_tile = atomicAdd(ctr, 1u);
-    __syncthreads();
-    const long long t = s_tile;
-    __syncthreads();                                 // s_tile is read before the next claim
+    if (!fixed) {
+      if (threadIdx.x == 0) s_tile = atomicAdd(ctr, 1u);
+      __syncthreads();
+    }
+    const long long t = fixed ? (long long)blockIdx.x : (long long)s_tile;
+    if (!fixed) __syncthreads();                     // s_tile is read before the next claim
     if (t >= n_tiles) break;
     T xs[U];
 #pragma unroll
@@ -588,12 +596,13 @@ onesweep_kernel(const T* in, T* out, unsigned* out_ids, unsigned id_mask, long l
       if (out_ids) out_ids[i] = (unsigned)x & id_mask;
       else out[i] = x;
     }
+    if (fixed) return;
   }
   for (; !s_copy;) {
-    if (threadIdx.x == 0) s_tile = atomicAdd(ctr, 1u);
+    if (!fixed && threadIdx.x == 0) s_tile = atomicAdd(ctr, 1u);
     for (int k = threadIdx.x; k < kOsWarps * (int)BINS; k += kOsThreads) (&cnt[0][0])[k] = 0;
     __syncthreads();
-    const long long t = s_tile;
+    const long long t = fixed ? (long long)blockIdx.x : (long long)s_tile;
     if (t >= n_tiles) break;                         // block-uniform
     const long long b0 = t * TILE + (long long)w * 32 * U;
     T xs[U];
@@ -703,6 +712,7 @@ onesweep_kernel(const T* in, T* out, unsigned* out_ids, unsigned id_mask, long l
         else out[pos] = x;
       }
     }
+    if (fixed) return;
     __syncthreads();                                 // before the next tile reuses cnt, s_off
   }
   if (threadIdx.x == 0) {
@@ -1126,7 +1136,8 @@ inline size_t place_smem_bytes(int rows, int tiles_x) {
 __global__ void __launch_bounds__(kPlaceThreads, 8)
 place_kernel(const u64* runs, const long long* n_runs, long long cap, const unsigned* row_runs,
              int rows, int tiles_x, const unsigned* ranges, const long long* K, unsigned* ids,
-             u64* state, unsigned* ctr, unsigned epoch, unsigned* status, unsigned spin_limit) {
+             u64* state, unsigned* ctr, unsigned epoch, unsigned* status, unsigned spin_limit,
+             unsigned resident) {
   pdl_prologue();
   extern __shared__ __align__(16) unsigned place_sm[];
   unsigned* s_rs = place_sm;                                  // [rows + 1] first run of a row
@@ -1163,9 +1174,12 @@ place_kernel(const u64* runs, const long long* n_runs, long long cap, const unsi
   }
   __syncthreads();
   const unsigned n_chunks = s_cs[rows];
+  // chunks that are all resident at once need no claims (as the radix passes' tiles)
+  const bool fixed = n_chunks <= resident;
+  if (fixed && blockIdx.x >= n_chunks) return;
   for (;;) {
     if (threadIdx.x == 0) {
-      const unsigned c = atomicAdd(ctr, 1u);
+      const unsigned c = fixed ? blockIdx.x : atomicAdd(ctr, 1u);
       unsigned y = 0;
       if (c < n_chunks) {                            // the row with s_cs[y] <= c < s_cs[y + 1]
         int lo = 0, hi = rows;
@@ -1270,6 +1284,7 @@ place_kernel(const u64* runs, const long long* n_runs, long long cap, const unsi
         if ((long long)pos < cap) ids[pos] = rid[q];
       }
     }
+    if (fixed) return;
     __syncthreads();                                 // before the next chunk reuses the arrays
   }
   if (threadIdx.x == 0) {
@@ -1287,14 +1302,15 @@ abcd_status launch_onesweep(abcd_ctx* ctx, cudaStream_t st, int bits, bool match
                             const unsigned* krange) {
   const unsigned epoch = ++ctx->os_epoch;
   const unsigned spin = ctx->wait_limit;
+  const unsigned resident = 2u * (unsigned)ctx->num_sms;    // the kernel's launch bounds
 #define ABCD_PASS(B)                                                                              \
   case B:                                                                                         \
     e = match ? launch_pdl(onesweep_kernel<T, B, true>, dim3(G), dim3(kOsThreads), 0, st, src, dst, \
                            ids, id_mask, n_static, n_dev, cap, shift, gh, ctx->ws.os_state, ctr,   \
-                           epoch, ctx->ws.status, spin, withhold, krange)                          \
+                           epoch, ctx->ws.status, spin, withhold, krange, resident)                \
               : launch_pdl(onesweep_kernel<T, B, false>, dim3(G), dim3(kOsThreads), 0, st, src,    \
                            dst, ids, id_mask, n_static, n_dev, cap, shift, gh, ctx->ws.os_state,   \
-                           ctr, epoch, ctx->ws.status, spin, withhold, krange);                    \
+                           ctr, epoch, ctx->ws.status, spin, withhold, krange, resident);          \
     break;
   cudaError_t e = cudaSuccess;
   switch (bits) {
@@ -1527,6 +1543,9 @@ extern "C" abcd_status abcd_bin_sort(abcd_ctx* ctx, const abcd_projected* proj, 
     const unsigned epoch = ++ctx->os_epoch;
     const int Gp = (int)std::max<long long>(1, std::min<long long>(max_chunks, 8LL * ctx->num_sms));
     const size_t psm = place_smem_bytes(tiles_y, tiles_x);
+    // CTAs that fit on the SMs at once: the launch bounds' eight, or what shared memory allows
+    const unsigned resident = (unsigned)ctx->num_sms *
+                              (unsigned)std::max<size_t>(1, std::min<size_t>(8, (200u << 10) / (psm + 2048)));
     {
       const cudaError_t e2 = ensure_smem(ctx, (const void*)place_kernel, psm);
       if (e2 != cudaSuccess) return fail(ctx, ABCD_ERR_CUDA, "place smem: %s", cudaGetErrorString(e2));
@@ -1537,7 +1556,7 @@ extern "C" abcd_status abcd_bin_sort(abcd_ctx* ctx, const abcd_projected* proj, 
                                    (const unsigned*)ctx->ws.row_runs, tiles_y, tiles_x,
                                    (const unsigned*)out->ranges, (const long long*)out->count,
                                    (unsigned*)out->ids, ctx->ws.os_state, ctx->ws.os_ctr + 4, epoch,
-                                   ctx->ws.status, ctx->wait_limit));
+                                   ctx->ws.status, ctx->wait_limit, resident));
   }
   int id_bits = 1;
   while ((1LL << id_bits) < n) ++id_bits;
