@@ -41,7 +41,7 @@ __device__ __forceinline__ float adam_one(float& th, float g, float& m, float& v
 // One thread per group of four consecutive elements of one array (float4 loads and stores when
 // the array allows, else scalar), grid-stride over the groups of the five arrays.
 __global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamArgs a) {
-  pdl_prologue();
+  pdl_wait();
   const unsigned total = a.gstart[5];
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
     int k = 0;

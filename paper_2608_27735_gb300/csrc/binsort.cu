@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kRankThreads)
 rank_sort_kernel(const float* depth, const int* radius, const float2* uv, int n, int per,
                  int tiles_x, int tiles_y, u64* sorted, int4* rects, unsigned* rows_zero,
                  int rows_words, int* diff_zero, int diff_cells) {
-  pdl_prologue();
+  pdl_wait();
   extern __shared__ __align__(16) unsigned s_key[];  // [n rounded up to 4], all ones past n
   clear_rows(rows_zero, rows_words, diff_zero, diff_cells);
   const int first = blockIdx.x * per, quads = (n + 3) / 4;
@@ -291,7 +291,7 @@ template <bool RUNS>
 __global__ void __launch_bounds__(256)
 tile_rows_kernel(const float2* uv, const float4* co, const int4* rects, int n, int tiles_x,
                  int tiles_y, float alpha_min, unsigned* counts, int* diff, unsigned* row_runs) {
-  pdl_prologue();
+  pdl_wait();
   extern __shared__ int sdiff[];
   const int W1 = tiles_x + 1;
   const int cells = W1 * (tiles_y + 1);
@@ -542,7 +542,7 @@ onesweep_kernel(const T* in, T* out, unsigned* out_ids, unsigned id_mask, long l
                 const long long* n_dev, long long cap, int shift, const unsigned* gh, u64* state,
                 unsigned* ctr, unsigned epoch, unsigned* status, unsigned spin_limit,
                 long long withhold, const unsigned* krange, unsigned resident) {
-  pdl_prologue();
+  pdl_wait();
   constexpr unsigned BINS = 1u << BITS, MASK = BINS - 1;
   constexpr int U = 64 / (int)sizeof(T);          // items per lane: 64 bytes in flight
   constexpr int TILE = kOsThreads * U;
@@ -726,7 +726,7 @@ onesweep_kernel(const T* in, T* out, unsigned* out_ids, unsigned id_mask, long l
 __global__ void __launch_bounds__(256)
 count_kernel(const u64* sorted, int n, const unsigned* counts, unsigned long long* block_sums,
              int G, long long* count, long long cap, unsigned* status, unsigned* ticket) {
-  pdl_prologue();
+  pdl_wait();
   long long lo, hi;
   block_range(n, G, &lo, &hi);
   unsigned long long s = 0;
@@ -776,7 +776,7 @@ count_kernel(const u64* sorted, int n, const unsigned* counts, unsigned long lon
 __global__ void __launch_bounds__(1024)
 ranges_from_diff_kernel(int* diff, int tiles_x, int tiles_y, long long cap, unsigned* ranges,
                         SortPasses tp, unsigned* gh) {
-  pdl_prologue();
+  pdl_wait();
   __shared__ unsigned dh[4][kRadixBins];
   for (int k = threadIdx.x; k < 4 * kRadixBins; k += blockDim.x) (&dh[0][0])[k] = 0u;
   const int W1 = tiles_x + 1;
@@ -833,7 +833,7 @@ __global__ void __launch_bounds__(1024)
 ranges_order_kernel(const int* diff, int tiles_x, int tiles_y, long long cap, unsigned* ranges,
                     unsigned* tile_order, SortPasses tp, unsigned* gh, const unsigned* row_runs,
                     long long* k_out, unsigned* status) {
-  pdl_prologue();
+  pdl_wait();
   extern __shared__ int sd[];              // [(tiles_x + 1) (tiles_y + 1)] cells, then [nt] keys
   __shared__ unsigned hist[kOrderBuckets];
   __shared__ unsigned dh[4][kRadixBins];   // digit counts of the tile sort's passes
@@ -967,7 +967,7 @@ __global__ void __launch_bounds__(kEmitThreads)
 emit_kernel(const u64* sorted, int n, const float2* uv, const float4* co, const int4* rects,
             const unsigned* counts, const unsigned long long* block_off, const long long* count,
             long long cap, int tiles_x, float alpha_min, int id_bits, T* pairs, int G) {
-  pdl_prologue();
+  pdl_wait();
   __shared__ Splat s_sp[kEmitThreads];
   __shared__ int4 s_q[kEmitThreads];
   __shared__ unsigned s_id[kEmitThreads];
@@ -1057,7 +1057,7 @@ __global__ void __launch_bounds__(kEmitThreads)
 emit_runs_kernel(const u64* sorted, int n, const float2* uv, const float4* co, const int4* rects,
                  const unsigned* counts, const unsigned long long* block_off, const long long* K,
                  long long cap, float alpha_min, u64* runs, int G) {
-  pdl_prologue();
+  pdl_wait();
   __shared__ Splat s_sp[kEmitThreads];
   __shared__ int4 s_q[kEmitThreads];
   __shared__ unsigned s_id[kEmitThreads];
@@ -1138,7 +1138,7 @@ place_kernel(const u64* runs, const long long* n_runs, long long cap, const unsi
              int rows, int tiles_x, const unsigned* ranges, const long long* K, unsigned* ids,
              u64* state, unsigned* ctr, unsigned epoch, unsigned* status, unsigned spin_limit,
              unsigned resident) {
-  pdl_prologue();
+  pdl_wait();
   extern __shared__ __align__(16) unsigned place_sm[];
   unsigned* s_rs = place_sm;                                  // [rows + 1] first run of a row
   unsigned* s_cs = s_rs + (rows + 1);                         // [rows + 1] first chunk of a row

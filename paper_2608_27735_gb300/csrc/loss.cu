@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(kQThreads, 3)
 ssim_fwd_kernel(const float* __restrict__ xin, const float* __restrict__ yin, int W, int H,
                 float lam, const Window win, float2* __restrict__ abc_ab, float* __restrict__ abc_c,
                 float* partials, unsigned* ticket, float* loss_out) {
-  pdl_prologue();
+  pdl_wait();
   extern __shared__ __align__(16) float sm[];
   float2* sXY = reinterpret_cast<float2*>(sm);           // [QR][QC]
   float2* vM = sXY + QR * QC;                            // [QH][QPM] windows of (x, y)
@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(kQThreads, 3)
 ssim_bwd_kernel(const float* __restrict__ xin, const float* __restrict__ yin, int W, int H,
                 float lam, const Window win, const float2* __restrict__ abc_ab,
                 const float* __restrict__ abc_c, float* __restrict__ grad) {
-  pdl_prologue();
+  pdl_wait();
   extern __shared__ __align__(16) float sm[];
   float2* sAB = reinterpret_cast<float2*>(sm);             // [QR][QC]
   float* sC = reinterpret_cast<float*>(sAB + QR * QC);     // [QR][QC]

@@ -368,7 +368,7 @@ template <int DEG>
 __global__ void __launch_bounds__(kProjThreads)
 project_bwd_kernel(Params p, int n, Cam cam, Opts op, SHConst K, const float* grad2d,
                    Grads out) {
-  pdl_prologue();
+  pdl_wait();
   constexpr int P = ShLayout<DEG>::P;
   __shared__ float s_sh[kProjThreads / 32][32 * P];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;

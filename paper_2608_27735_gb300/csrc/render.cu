@@ -447,7 +447,7 @@ __device__ __forceinline__ void fetch_group(const FwdArgs& a, const unsigned (&g
 // registers and gave 61 and 207 us; 32 positions per group 29 us and 72 us.  24 CTAs per SM (80
 // registers, no spills) against 28: 61 against 63 us and 189 against 199 us.
 __global__ void __launch_bounds__(kSubThreads, 24) render_fwd_kernel(const __grid_constant__ FwdArgs a) {
-  pdl_prologue();
+  pdl_wait();
   __shared__ RawGroup raw;
   __shared__ float4 s_co[kFwdGroup];
   __shared__ float4 s_m[kFwdGroup];
@@ -787,7 +787,7 @@ __device__ __forceinline__ void bwd_chunk(const BwdArgs& a, int blk, int start, 
 // and 427 us; staging through asynchronous copies 100, 80 and 467 us (more shared-memory traffic).
 // 20 CTAs per SM leave 96 registers, so nothing spills; 16 CTAs 94, 76 and 434 us.
 __global__ void __launch_bounds__(kSubThreads, 20) render_bwd_kernel(BwdArgs a) {
-  pdl_prologue();
+  pdl_wait();
   __shared__ float4 s_co[kGroup + kBwdUnroll - 1];
   __shared__ float4 s_m[kGroup + kBwdUnroll - 1];
   __shared__ float4 s_rgb[kGroup + kBwdUnroll - 1];
