@@ -91,13 +91,14 @@ constexpr int kRenderSubPerTile = 4;      // render CTAs (8x8 pixel blocks) per 
 // holding slots meanwhile.  That pays only where this grid is short and the next one's CTAs are
 // few and alike: project_fwd -> keys_rects -> sort_digits -> the first radix pass, zero_kernel
 // (whose own early start keeps the render kernels' CTAs from becoming resident before the kernel
-// ahead of it has ended), and the kernels outside the step.
+// ahead of it has ended), composite_packed_kernel (19.6 against 19.8 us), and the one-CTA and
+// whole-loss kernels outside the step.
 //
 // The step with every trigger early, every one late, and as built (us): 2,000 Gaussians at 128x128
 // 103 / 96 / 96; 20,000 at 640x480 171 / 160 / 160; 33,000 at 1001x667 243 / 242 / 239; 100,000 at
 // 1237x822 342 / 346 / 342; forward and backward of 2M at 1080p 2,188 / 2,101 / 2,105.  One call:
 // the loss at 1080p 154 -> 136 and at 1237x822 61.4 -> 58.5, abcd_bin_sort of 2M 1,066 -> 1,032,
-// of 20,000 58 -> 54.
+// of 20,000 58 -> 54, the folds 35.5 -> 34.5, the visibility pass 26.3 -> 25.8.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_prologue() {
   pdl_wait();

@@ -135,7 +135,7 @@ template <int PIX, bool F16>
 __global__ void __launch_bounds__(256)
 composite_kernel(const __grid_constant__ LayerTable lt, int nf, int nb, long long groups,
                  void* Fout, void* Bout, int out_f16) {
-  pdl_prologue();
+  pdl_wait();
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < groups;
        g += (long long)gridDim.x * blockDim.x) {
     float acc[4 * PIX];
@@ -321,7 +321,7 @@ composite_packed_kernel(const __grid_constant__ PackedTable pt, int nf, int nb, 
 __global__ void __launch_bounds__(kPackedThreads)
 fold_packed_kernel(const __grid_constant__ PackedTable pt, int n, int width, int height,
                    int tiles_x, const float4* acc_in, float4* acc_out, uint2* out16) {
-  pdl_prologue();
+  pdl_wait();
   __shared__ int s_map[kMaxLayers], s_list[kMaxLayers], s_count;
   const int tile = blockIdx.x;
   const int unit = threadIdx.x;
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(kPackedThreads, 10)
 visibility_kernel(const __grid_constant__ VisTable vt, int count, int L, int width, int height,
                   int tiles_x, int n_tiles, unsigned long long* sums, unsigned* ticket,
                   double* visible, double* coverage) {
-  pdl_prologue();
+  pdl_wait();
   __shared__ unsigned long long s_sum[2][kMaxLayers];
   __shared__ int s_map[kMaxLayers];
   __shared__ int s_list[kMaxLayers];
