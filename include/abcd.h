@@ -129,7 +129,9 @@ abcd_status abcd_set_wait_limit(abcd_ctx* ctx, unsigned polls);
 /* Test hook for the bounded waits: in the next abcd_bin_sort call, look-back tile `tile` (2048
  * keys) of the first pass of the depth sort publishes nothing, so the waits of the tiles after
  * it run out (after the wait limit).  -1 (the default) turns it off; it turns itself off after
- * that pass. */
+ * that pass.  While it is set, blocks of any size are sorted by the radix passes (small ones are
+ * otherwise ordered by counting, which waits for nothing); a tile past the last one withholds
+ * nothing. */
 abcd_status abcd_test_withhold_lookback(abcd_ctx* ctx, long long tile);
 
 /* ---- the hot path (Section 2: one step renders only the active block) ----------------- */

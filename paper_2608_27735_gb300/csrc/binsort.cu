@@ -94,8 +94,8 @@ __device__ __forceinline__ void clear_rows(unsigned* rows_zero, int rows_words, 
 // it.  n^2 comparisons, but one launch where the digit counts and four radix passes are five.
 // Every CTA holds all keys in shared memory and places `per` items, 256 / per threads each.  Also
 // the tile rectangles.  Up to kRankMax items, where the comparisons overtake the passes:
-// abcd_bin_sort 35 against 50 us with 1,000 Gaussians, 38 against 53 with 2,000, 50 against 57
-// with 4,000, 57 against 61 with 6,000, 80 against 62 with 8,192.
+// abcd_bin_sort 31 against 40 us with 1,000 Gaussians, 32 against 42 with 2,000, 37 against 49
+// with 4,000, 45 against 51 with 6,000; with 8,192 the counting took 18 us more than the passes.
 constexpr int kRankMax = 6144;
 constexpr int kRankThreads = 256;
 
@@ -568,10 +568,11 @@ onesweep_kernel(const T* in, T* out, unsigned* out_ids, unsigned id_mask, long l
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const KeyMap km = key_map(krange);
-  // Tiles that are all resident at once need no claims: CTA b takes tile b (and the tiles it
-  // waits for are running, or are started as soon as another kernel's CTA ends).  That saves
-  // three round trips per pass (the claim, the claim that finds nothing left, the counters'
-  // reset): a pass over 100,000 keys 12.0 -> 10.2 us, abcd_bin_sort 93 -> 82 us there.
+  // Tiles that are all resident at once need no claims: CTA b takes tile b.  The tiles it waits
+  // for have lower CTA indices and were started before it; the wait's bound also covers a start
+  // in another order with the SMs full of other streams' work.  That saves three round trips per
+  // pass (the claim, the claim that finds nothing left, the counters' reset): a pass over 100,000
+  // keys 12.0 -> 10.2 us, abcd_bin_sort 93 -> 82 us there.
   const bool fixed = n_tiles <= (long long)resident;
   if (fixed && blockIdx.x >= n_tiles) return;
   while (s_copy) {                                   // block-uniform (set before the scan's barriers)

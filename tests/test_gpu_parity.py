@@ -973,6 +973,56 @@ def test_small_blocks_order_as_the_radix_sort(ctx, n, depths):
     assert n < 64 or got[0][0] > 0
 
 
+@pytest.mark.parametrize("over", [0, 1])
+def test_bin_sort_at_the_resident_limit(over):
+    """The largest sort whose radix tiles and placement chunks are taken by CTA index, and one
+    Gaussian more (they are claimed): one tile lists every Gaussian in stable depth order."""
+    n = 2 * torch.cuda.get_device_properties(0).multi_processor_count * 2048 + over
+    ctx = ab.Context()
+    ctx.reserve(n, n, 256)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    proj = ab.Projected.alloc(n)
+    proj.uv.fill_(8.0)
+    proj.conic_opacity.copy_(torch.tensor([0.01, 0.0, 0.01, 0.9], device="cuda").expand(n, 4))
+    proj.depth.copy_(torch.round(1.0 + 2000.0 * torch.rand(n, generator=g, device="cuda"), decimals=2))
+    proj.radius.fill_(30)
+    tiles = ab.Tiles.alloc(n, 16, 16)
+    ab.abcd_bin_sort(ctx, proj, n, ab.camera(sg.look_at((0.0, -5.0, 0.0), np.zeros(3), 16, 16)), tiles)
+    ctx.sync()
+    assert int(tiles.count.item()) == n
+    assert torch.equal(tiles.ids[:n].long(), torch.sort(proj.depth, stable=True).indices)
+
+
+def test_bin_sort_on_several_streams_at_once():
+    """Sorts whose CTAs do not fit on the GPU together: each gives the lists it gives alone."""
+    n, W, H, count = 60_000, 640, 480, 6
+    g = torch.Generator(device="cuda").manual_seed(11)
+    proj = ab.Projected.alloc(n)
+    proj.uv.copy_(torch.rand(n, 2, generator=g, device="cuda") * torch.tensor([W * 1.0, H * 1.0], device="cuda"))
+    proj.conic_opacity.copy_(torch.tensor([0.01, 0.0, 0.01, 0.9], device="cuda").expand(n, 4))
+    proj.depth.copy_(1.0 + 9.0 * torch.rand(n, generator=g, device="cuda"))
+    proj.radius.fill_(30)
+    cam = ab.camera(sg.look_at((0.0, -5.0, 0.0), np.zeros(3), W, H))
+    torch.cuda.synchronize()
+    ctxs = [ab.Context(stream=torch.cuda.Stream()) for _ in range(count)]
+    tiles = [ab.Tiles.alloc(2_000_000, W, H) for _ in range(count)]
+    for c in ctxs:
+        c.reserve(n, 2_000_000, W * H)
+    torch.cuda.synchronize()
+    ab.abcd_bin_sort(ctxs[0], proj, n, cam, tiles[0])
+    ctxs[0].sync()
+    K = int(tiles[0].count.item())
+    ids, ranges = tiles[0].ids[:K].clone(), tiles[0].ranges.clone()
+    torch.cuda.synchronize()
+    for _ in range(8):
+        for c, t in zip(ctxs, tiles):
+            ab.abcd_bin_sort(c, proj, n, cam, t)
+    for c, t in zip(ctxs, tiles):
+        c.sync()
+        assert int(t.count.item()) == K > 0
+        assert torch.equal(t.ids[:K], ids) and torch.equal(t.ranges, ranges)
+
+
 def test_invalid_arguments_rejected(ctx):
     cam = ab.abcd_camera()
     cam.width = 0
