@@ -89,10 +89,9 @@ constexpr int kRenderSubPerTile = 4;      // render CTAs (8x8 pixel blocks) per 
 // resident early and wait; the wait's end then finds them where there was room at that moment: many on
 // some SMs and few on others, in launch order (the longest render walks next to each other), and
 // holding slots meanwhile.  That pays only where this grid is short and the next one's CTAs are
-// few and alike: project_fwd -> keys_rects -> sort_digits -> the first radix pass, zero_kernel
-// (whose own early start keeps the render kernels' CTAs from becoming resident before the kernel
-// ahead of it has ended), composite_packed_kernel (19.6 against 19.8 us), and the one-CTA and
-// whole-loss kernels outside the step.
+// few and alike: project_fwd -> keys_rects -> sort_digits -> the first radix pass, zero_kernel (a
+// short kernel ahead of the render kernels), composite_packed_kernel (19.6 against 19.8 us), and
+// the one-CTA and whole-loss kernels outside the step.
 //
 // The step with every trigger early, every one late, and as built (us): 2,000 Gaussians at 128x128
 // 103 / 96 / 96; 20,000 at 640x480 171 / 160 / 160; 33,000 at 1001x667 243 / 242 / 239; 100,000 at
@@ -181,8 +180,23 @@ Cam make_cam(const abcd_camera* c, const abcd_render_opts* o);
 Opts make_opts(const abcd_render_opts* o);
 void sh_constants(SHConst* out);
 
-// translation-unit entry points used by the composite calls
+// Entry points the composite calls use: the public calls with what the call before them can take
+// over.  loss_launch also clears zero[0, zero_n) when its gradient kernel runs (floats, 16-byte
+// aligned); bin_sort also clears zero_word, and says so in *zeroed; the render calls skip the
+// clear of the checkpoint count / of grad2d when it has been done.
 abcd_status loss_launch(abcd_ctx* ctx, const float* out_rgba, const float* gt_rgb, int width,
-                        int height, float lambda_ssim, float* loss_out, float* dL_dout);
+                        int height, float lambda_ssim, float* loss_out, float* dL_dout,
+                        float* zero = nullptr, long long zero_n = 0);
+abcd_status bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n, const abcd_camera* cam,
+                     const abcd_render_opts* opts, abcd_tiles* out, unsigned* zero_word, bool* zeroed);
+abcd_status render_composite_fwd(abcd_ctx* ctx, const abcd_camera* cam, const abcd_render_opts* opts,
+                                 const abcd_projected* proj, const abcd_tiles* tiles, const void* F,
+                                 const void* B, int fb_dtype, const float* bg, float* out_rgba,
+                                 abcd_fwd_state* state, void* refresh_f16, bool count_cleared);
+abcd_status render_backward(abcd_ctx* ctx, const abcd_camera* cam, const abcd_render_opts* opts,
+                            const abcd_projected* proj, const abcd_tiles* tiles, const void* F,
+                            const void* B, int fb_dtype, const float* bg,
+                            const abcd_fwd_state* state, const float* dL_dout, int n, float* grad2d,
+                            bool grad_cleared);
 
 }  // namespace abcd

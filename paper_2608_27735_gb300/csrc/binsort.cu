@@ -81,9 +81,10 @@ __device__ __forceinline__ u64 depth_item(float2 m, int r, float z, int i, int t
 
 // Zeroes the words the binning adds to: per-row run counts and the tile rows' difference array
 // (here rather than by a memset, which would end the programmatic overlap of the launches before
-// and after it).
+// and after it); and a word for the caller.
 __device__ __forceinline__ void clear_rows(unsigned* rows_zero, int rows_words, int* diff_zero,
-                                           int diff_cells) {
+                                           int diff_cells, unsigned* zero_word) {
+  if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0u;
   if (blockIdx.x == 0)
     for (int k = threadIdx.x; k < rows_words; k += blockDim.x) rows_zero[k] = 0u;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < diff_cells; k += gridDim.x * blockDim.x)
@@ -102,10 +103,10 @@ constexpr int kRankThreads = 256;
 __global__ void __launch_bounds__(kRankThreads)
 rank_sort_kernel(const float* depth, const int* radius, const float2* uv, int n, int per,
                  int tiles_x, int tiles_y, u64* sorted, int4* rects, unsigned* rows_zero,
-                 int rows_words, int* diff_zero, int diff_cells) {
+                 int rows_words, int* diff_zero, int diff_cells, unsigned* zero_word) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned s_key[];  // [n rounded up to 4], all ones past n
-  clear_rows(rows_zero, rows_words, diff_zero, diff_cells);
+  clear_rows(rows_zero, rows_words, diff_zero, diff_cells, zero_word);
   const int first = blockIdx.x * per, quads = (n + 3) / 4;
   constexpr int kBatch = 8;                          // items a thread has in flight
   for (int b0 = 0; b0 < 4 * quads; b0 += kBatch * kRankThreads) {
@@ -167,14 +168,14 @@ __global__ void keys_rects_kernel(const float* depth, const int* radius, const f
                                   int tiles_x, int tiles_y, u64* items, int4* rects,
                                   unsigned* gh_zero, int gh_words, unsigned* rows_zero,
                                   int rows_words, int* diff_zero, int diff_cells, unsigned* krange,
-                                  unsigned* krange_next) {
+                                  unsigned* krange_next, unsigned* zero_word) {
   pdl_prologue();
   if (blockIdx.x == 0) {                  // the radix sorts' digit counts start from zero
     for (int k = threadIdx.x; k < gh_words; k += blockDim.x) gh_zero[k] = 0u;
     // the key range words of the next call (two pairs used in turn, so no memset is needed)
     if (threadIdx.x < 2) krange_next[threadIdx.x] = 0u;
   }
-  clear_rows(rows_zero, rows_words, diff_zero, diff_cells);
+  clear_rows(rows_zero, rows_words, diff_zero, diff_cells, zero_word);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   bool vis = false;
   unsigned key = 0xFFFFFFFFu;
@@ -1378,6 +1379,12 @@ using namespace abcd;
 extern "C" abcd_status abcd_bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n,
                                      const abcd_camera* cam, const abcd_render_opts* opts,
                                      abcd_tiles* out) {
+  return bin_sort(ctx, proj, n, cam, opts, out, nullptr, nullptr);
+}
+
+abcd_status abcd::bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n, const abcd_camera* cam,
+                           const abcd_render_opts* opts, abcd_tiles* out, unsigned* zero_word,
+                           bool* zeroed) {
   if (!ctx) return ABCD_ERR_INVALID_ARG;
   if (!has_workspace(ctx)) return fail(ctx, ABCD_ERR_WORKSPACE, "abcd_bin_sort: no workspace");
   if (!proj || !cam || !out || n < 0 || cam->width <= 0 || cam->height <= 0)
@@ -1429,6 +1436,7 @@ extern "C" abcd_status abcd_bin_sort(abcd_ctx* ctx, const abcd_projected* proj, 
   // the passes count from the tile (row) bits' lowest, the sorts' own from the items' field
   const SortPasses tile_passes = make_passes(0, by_runs ? row_bits : tile_bits);
   unsigned* tile_gh = ctx->ws.os_gh + 4 * kRadixBins;
+  if (zeroed) *zeroed = zero_word != nullptr;        // (by the first kernel, whichever it is)
   // up to kRankMax Gaussians the depth order comes from one kernel (unless the test hook asks for
   // a look-back wait that runs out), and everything runs on the context's stream
   const bool rank = n <= kRankMax && ctx->withhold_tile < 0;
@@ -1444,7 +1452,7 @@ extern "C" abcd_status abcd_bin_sort(abcd_ctx* ctx, const abcd_projected* proj, 
                                      smem, ctx->stream, (const float*)proj->depth,
                                      (const int*)proj->radius, (const float2*)proj->uv, n, per,
                                      tiles_x, tiles_y, by_depth, ctx->ws.rects, ctx->ws.row_runs,
-                                     by_runs ? tiles_y : 0, ctx->ws.diff, cells))))
+                                     by_runs ? tiles_y : 0, ctx->ws.diff, cells, zero_word))))
       return s;
   } else {
     if ((s = check_launch(ctx, "keys_rects_kernel",
@@ -1455,7 +1463,7 @@ extern "C" abcd_status abcd_bin_sort(abcd_ctx* ctx, const abcd_projected* proj, 
                                      (const float2*)proj->uv, n, tiles_x, tiles_y, ctx->ws.dsort[0],
                                      ctx->ws.rects, ctx->ws.os_gh, 2 * 4 * kRadixBins,
                                      ctx->ws.row_runs, by_runs ? tiles_y : 0, ctx->ws.diff, cells,
-                                     krange, krange_next))))
+                                     krange, krange_next, zero_word))))
       return s;
     ++ctx->krange_parity;                            // the next call's pair is being cleared
     // the tile rows and ranges only need the rectangles: they run on the side stream while the

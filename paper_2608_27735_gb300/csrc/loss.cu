@@ -516,8 +516,17 @@ ssim_fwd_kernel(const float* __restrict__ xin, const float* __restrict__ yin, in
 __global__ void __launch_bounds__(kQThreads, 3)
 ssim_bwd_kernel(const float* __restrict__ xin, const float* __restrict__ yin, int W, int H,
                 float lam, const Window win, const float2* __restrict__ abc_ab,
-                const float* __restrict__ abc_c, float* __restrict__ grad) {
+                const float* __restrict__ abc_c, float* __restrict__ grad,
+                float* __restrict__ zero, long long zero_n) {
   pdl_wait();
+  // clears the caller's buffer on the side (the render backward's gradient sums: a launch less, and
+  // the stores hide behind the windows)
+  if (zero) {
+    const long long cta = q_block_index(), ctas = (long long)gridDim.x * gridDim.y * gridDim.z;
+    for (long long i = cta * kQThreads + threadIdx.x; i < zero_n / 4; i += ctas * kQThreads)
+      reinterpret_cast<float4*>(zero)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (cta == 0 && threadIdx.x < zero_n % 4) zero[zero_n / 4 * 4 + threadIdx.x] = 0.f;
+  }
   extern __shared__ __align__(16) float sm[];
   float2* sAB = reinterpret_cast<float2*>(sm);             // [QR][QC]
   float* sC = reinterpret_cast<float*>(sAB + QR * QC);     // [QR][QC]
@@ -647,7 +656,8 @@ dim3 loss_grid(int width, int height) {
 }  // namespace
 
 abcd_status loss_launch(abcd_ctx* ctx, const float* out_rgba, const float* gt_rgb, int width,
-                        int height, float lambda_ssim, float* loss_out, float* dL_dout) {
+                        int height, float lambda_ssim, float* loss_out, float* dL_dout, float* zero,
+                        long long zero_n) {
   if (!has_workspace(ctx)) return fail(ctx, ABCD_ERR_WORKSPACE, "abcd_loss: no workspace");
   if (!out_rgba || !gt_rgb || width <= 0 || height <= 0 || !(lambda_ssim >= 0.f && lambda_ssim <= 1.f))
     return fail(ctx, ABCD_ERR_INVALID_ARG, "abcd_loss: bad arguments");
@@ -672,7 +682,8 @@ abcd_status loss_launch(abcd_ctx* ctx, const float* out_rgba, const float* gt_rg
   return check_launch(ctx, "ssim_bwd_kernel",
                       launch_pdl(ssim_bwd_kernel, grid, dim3(kQThreads), smem_b, ctx->stream, out_rgba,
                                  gt_rgb, width, height, lambda_ssim, win,
-                                 (const float2*)ctx->ws.ssim_ab, (const float*)ctx->ws.ssim_c, dL_dout));
+                                 (const float2*)ctx->ws.ssim_ab, (const float*)ctx->ws.ssim_c, dL_dout, zero,
+                                 zero_n));
 }
 
 }  // namespace abcd

@@ -844,13 +844,12 @@ bool proj_ok(const abcd_projected* p) {
 
 using namespace abcd;
 
-extern "C" abcd_status abcd_render_composite_fwd(abcd_ctx* ctx, const abcd_camera* cam,
-                                                 const abcd_render_opts* opts,
-                                                 const abcd_projected* proj,
-                                                 const abcd_tiles* tiles, const void* F,
-                                                 const void* B, int fb_dtype, const float* bg,
-                                                 float* out_rgba, abcd_fwd_state* state,
-                                                 void* refresh_f16) {
+abcd_status abcd::render_composite_fwd(abcd_ctx* ctx, const abcd_camera* cam,
+                                       const abcd_render_opts* opts, const abcd_projected* proj,
+                                       const abcd_tiles* tiles, const void* F, const void* B,
+                                       int fb_dtype, const float* bg, float* out_rgba,
+                                       abcd_fwd_state* state, void* refresh_f16,
+                                       bool count_cleared) {
   if (!ctx) return ABCD_ERR_INVALID_ARG;
   if (!cam || cam->width <= 0 || cam->height <= 0 || !tiles || !tiles->ids || !tiles->ranges)
     return fail(ctx, ABCD_ERR_INVALID_ARG, "abcd_render_composite_fwd: bad camera or tiles");
@@ -882,8 +881,10 @@ extern "C" abcd_status abcd_render_composite_fwd(abcd_ctx* ctx, const abcd_camer
   a.ckpt = nullptr; a.ck_items = nullptr; a.ck_count = nullptr; a.ck_first = nullptr;
   a.ck_cap = 0;
   if (state && ckpt_ok(ctx, n_blocks)) {
-    const abcd_status z = zero_async(ctx, ctx->ws.ck_count, sizeof(unsigned), "checkpoint count clear");
-    if (z != ABCD_OK) return z;
+    if (!count_cleared) {
+      const abcd_status z = zero_async(ctx, ctx->ws.ck_count, sizeof(unsigned), "checkpoint count clear");
+      if (z != ABCD_OK) return z;
+    }
     a.ckpt = ctx->ws.ckpt; a.ck_items = ctx->ws.ck_items; a.ck_count = ctx->ws.ck_count;
     a.ck_first = ctx->ws.ck_first; a.ck_cap = ctx->ws.ck_cap;
     ctx->ck_state = state->A_T;
@@ -896,12 +897,22 @@ extern "C" abcd_status abcd_render_composite_fwd(abcd_ctx* ctx, const abcd_camer
                       launch_pdl(render_fwd_kernel, dim3(n_blocks), dim3(kSubThreads), 0, ctx->stream, a));
 }
 
-extern "C" abcd_status abcd_render_backward(abcd_ctx* ctx, const abcd_camera* cam,
-                                            const abcd_render_opts* opts,
-                                            const abcd_projected* proj, const abcd_tiles* tiles,
-                                            const void* F, const void* B, int fb_dtype,
-                                            const float* bg, const abcd_fwd_state* state,
-                                            const float* dL_dout, int n, float* grad2d) {
+extern "C" abcd_status abcd_render_composite_fwd(abcd_ctx* ctx, const abcd_camera* cam,
+                                                 const abcd_render_opts* opts,
+                                                 const abcd_projected* proj,
+                                                 const abcd_tiles* tiles, const void* F,
+                                                 const void* B, int fb_dtype, const float* bg,
+                                                 float* out_rgba, abcd_fwd_state* state,
+                                                 void* refresh_f16) {
+  return render_composite_fwd(ctx, cam, opts, proj, tiles, F, B, fb_dtype, bg, out_rgba, state,
+                              refresh_f16, false);
+}
+
+abcd_status abcd::render_backward(abcd_ctx* ctx, const abcd_camera* cam,
+                                  const abcd_render_opts* opts, const abcd_projected* proj,
+                                  const abcd_tiles* tiles, const void* F, const void* B,
+                                  int fb_dtype, const float* bg, const abcd_fwd_state* state,
+                                  const float* dL_dout, int n, float* grad2d, bool grad_cleared) {
   if (!ctx) return ABCD_ERR_INVALID_ARG;
   if (!cam || cam->width <= 0 || cam->height <= 0 || !tiles || !tiles->ids || !tiles->ranges)
     return fail(ctx, ABCD_ERR_INVALID_ARG, "abcd_render_backward: bad camera or tiles");
@@ -910,7 +921,7 @@ extern "C" abcd_status abcd_render_backward(abcd_ctx* ctx, const abcd_camera* ca
   if (!state || !state->A_T || !state->n_last || !dL_dout || n < 0 || (n > 0 && !grad2d))
     return fail(ctx, ABCD_ERR_INVALID_ARG, "abcd_render_backward: null state, gradient or output");
   if (n == 0) return ABCD_OK;
-  {
+  if (!grad_cleared) {
     const abcd_status z = zero_async(ctx, grad2d, sizeof(float) * 9 * (size_t)n, "grad2d clear");
     if (z != ABCD_OK) return z;
   }
@@ -942,6 +953,16 @@ extern "C" abcd_status abcd_render_backward(abcd_ctx* ctx, const abcd_camera* ca
   return check_launch(ctx, "render_bwd_kernel",
                       launch_pdl(render_bwd_kernel, dim3(a.n_item_ctas + n_blocks), dim3(kSubThreads),
                                  0, ctx->stream, a));
+}
+
+extern "C" abcd_status abcd_render_backward(abcd_ctx* ctx, const abcd_camera* cam,
+                                            const abcd_render_opts* opts,
+                                            const abcd_projected* proj, const abcd_tiles* tiles,
+                                            const void* F, const void* B, int fb_dtype,
+                                            const float* bg, const abcd_fwd_state* state,
+                                            const float* dL_dout, int n, float* grad2d) {
+  return render_backward(ctx, cam, opts, proj, tiles, F, B, fb_dtype, bg, state, dL_dout, n, grad2d,
+                         false);
 }
 
 // ---- packed layers (the cache's tile-sparse format): tile t of a layer is stored iff its

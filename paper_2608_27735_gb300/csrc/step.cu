@@ -5,6 +5,12 @@
 
 using namespace abcd;
 
+// The gradient sums (36 bytes per Gaussian) are cleared by the loss's gradient kernel up to this
+// size: a launch less in front of the render backward (steps of 2,000 to 100,000 Gaussians 1-2%
+// shorter with the checkpoint count's, 300,000 to 1M, 36 MB, 1-3%).  2M Gaussians' 72 MB hold
+// that kernel up longer than the launch costs (2,094 against 2,088 us forward and backward).
+static constexpr long long kRideBytes = 40LL << 20;
+
 extern "C" abcd_status abcd_backward(abcd_ctx* ctx, const abcd_gaussians* theta,
                                      const abcd_camera* cam, const abcd_render_opts* opts,
                                      const abcd_projected* proj, const abcd_tiles* tiles,
@@ -19,17 +25,20 @@ extern "C" abcd_status abcd_backward(abcd_ctx* ctx, const abcd_gaussians* theta,
   const long long npix = (long long)cam->width * cam->height;
   const float* g = dL_dout;
   abcd_status s;
+  bool cleared = false;                              // grad2d, by the loss's gradient kernel
   if (gt_rgb) {
+    const bool rides = theta->n > 0 && 36LL * theta->n <= kRideBytes;
     if (npix > ctx->max_pixels) return fail(ctx, ABCD_ERR_WORKSPACE, "abcd_backward: image exceeds workspace");
     if ((s = loss_launch(ctx, out_rgba, gt_rgb, cam->width, cam->height, lambda_ssim, loss_out,
-                         ctx->ws.dl_dout)))
+                         ctx->ws.dl_dout, rides ? ctx->ws.grad2d : nullptr, 9LL * theta->n)))
       return s;
+    cleared = rides;
     g = ctx->ws.dl_dout;
   } else if (!g) {
     return fail(ctx, ABCD_ERR_INVALID_ARG, "abcd_backward: need gt_rgb or dL_dout");
   }
-  if ((s = abcd_render_backward(ctx, cam, opts, proj, tiles, F, B, fb_dtype, bg, state, g,
-                                theta->n, ctx->ws.grad2d)))
+  if ((s = render_backward(ctx, cam, opts, proj, tiles, F, B, fb_dtype, bg, state, g, theta->n,
+                           ctx->ws.grad2d, cleared)))
     return s;
   return abcd_project_backward(ctx, theta, cam, opts, ctx->ws.grad2d, grads);
 }
@@ -48,9 +57,13 @@ extern "C" abcd_status abcd_train_step(abcd_ctx* ctx, abcd_gaussians* theta, abc
     return fail(ctx, ABCD_ERR_INVALID_ARG, "abcd_train_step: null argument");
   abcd_status s;
   if ((s = abcd_project(ctx, theta, cam, opts, proj))) return s;
-  if ((s = abcd_bin_sort(ctx, proj, theta->n, cam, opts, tiles))) return s;
-  if ((s = abcd_render_composite_fwd(ctx, cam, opts, proj, tiles, F, B, fb_dtype, bg, out_rgba,
-                                     state, nullptr)))
+  // the binning's first kernel also clears the render's checkpoint count, so no earlier forward's
+  // checkpoints are valid any more
+  bool cleared = false;
+  ctx->ck_state = nullptr;
+  if ((s = bin_sort(ctx, proj, theta->n, cam, opts, tiles, ctx->ws.ck_count, &cleared))) return s;
+  if ((s = render_composite_fwd(ctx, cam, opts, proj, tiles, F, B, fb_dtype, bg, out_rgba, state,
+                                nullptr, cleared)))
     return s;
   if ((s = abcd_backward(ctx, theta, cam, opts, proj, tiles, F, B, fb_dtype, bg, out_rgba, state,
                          gt_rgb, lambda_ssim, loss_out, nullptr, grads)))

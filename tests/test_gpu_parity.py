@@ -829,6 +829,37 @@ def test_train_step_matches_separate_calls(ctx, tiny):
         assert torch.allclose(a_, b_, rtol=1e-4, atol=1e-7)
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 63])
+def test_backward_clears_its_sums(ctx, tiny, n):
+    """abcd_backward from a target (its loss clears the gradient sums, any remainder of four) gives
+    what it gives from the loss's own gradient (a kernel clears them), up to the order of the
+    atomic sums, with the sums of an earlier, larger call in the workspace."""
+    case = Case(tiny, 1, fb=True)
+    H, W = case.cam.height, case.cam.width
+    r = run_forward(ctx, case)
+    gt = torch.from_numpy(sg.random_image(H, W, 3, seed=78)).cuda()
+    loss, full = torch.zeros(1, device="cuda"), ab.Gaussians.zeros_like(r["theta"])
+    ab.abcd_backward(ctx, r["theta"], r["cam"], None, r["proj"], r["tiles"], r["F"], r["B"], r["fbd"],
+                     None, r["out"], r["state"], gt, 0.2, loss, None, full)
+    theta = ab.Gaussians(*(t[:n].contiguous() for t in r["theta"].tensors()), r["theta"].sh_degree)
+    proj = ab.Projected.alloc(n)
+    ab.abcd_project(ctx, theta, r["cam"], None, proj)
+    ab.abcd_bin_sort(ctx, proj, n, r["cam"], r["tiles"])
+    ab.abcd_render_composite_fwd(ctx, r["cam"], None, proj, r["tiles"], r["F"], r["B"], r["fbd"], None,
+                                 r["out"], r["state"])
+    dl = torch.zeros(H, W, 3, device="cuda")
+    ab.abcd_loss(ctx, r["out"], gt, W, H, 0.2, loss, dl)
+    got = []
+    for target, grad in ((gt, None), (None, dl)):
+        grads = ab.Gaussians.zeros_like(theta)
+        ab.abcd_backward(ctx, theta, r["cam"], None, proj, r["tiles"], r["F"], r["B"], r["fbd"], None,
+                         r["out"], r["state"], target, 0.2, loss, grad, grads)
+        got.append(grads)
+    ctx.sync()
+    for a_, b_ in zip(got[0].tensors(), got[1].tensors()):
+        assert torch.allclose(a_, b_, rtol=1e-4, atol=1e-7)
+
+
 @pytest.mark.parametrize("seed,cam_idx", [(1001, 0), (1005, 1)])
 def test_full_step_matches_oracle(ctx, seed, cam_idx):
     """project -> bin/sort -> render + composite -> L1 + 0.2 D-SSIM -> backward, element-wise.
