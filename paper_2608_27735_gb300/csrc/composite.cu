@@ -221,6 +221,15 @@ struct PackedTable {
 
 constexpr int kPackedThreads = kTileThreads / 2;
 constexpr int kPackedInFlight = 8;
+// Sides of up to kShortLayers layers are folded without the list (F, then B, by 128 threads, no
+// shared memory): with few layers its barriers cost more than its loads gain.  At 1210x883, a
+// tenth and nine tenths of the tiles stored: 3 layers 9.4 -> 6.9 and 12.6 -> 8.7 us; 9 layers 10.2
+// -> 8.7, half stored 14.6 -> 11.5; 13 layers, a third stored, 14.3 -> 12.3.  Without the line 24
+// layers take 18.6 against 17.0 us and 64 (a tenth stored) 33 against 19.  Four loads in flight
+// and 12 CTAs per SM (40 registers): eight take 8.2 us for 3 layers, 16 CTAs spill.
+constexpr int kShortLayers = 8;
+constexpr int kShortInFlight = 4;
+constexpr int kShortCtas = 12;
 
 // The positions k in [k0, k1) with s_map[k] >= 0, in order, into s_list, and how many into
 // *s_count; warp 0 of the calling threads (thread: 0 for the first) compacts with ballots, and
@@ -282,35 +291,73 @@ __device__ __forceinline__ void store_pixel_out(void* out, int f16, long long p,
   }
 }
 
-// F by the first half of the CTA and B by the second, each over the list of the layers that
-// store the tile.
-__global__ void __launch_bounds__(2 * kPackedThreads)
+// Layers [k0, k1) folded into acc without the list: each thread reads the tile's map entries
+// itself, then has the stored layers' loads in flight together, kShortInFlight layers at a time.
+__device__ __forceinline__ void fold_short(const PackedTable& pt, int k0, int k1, int tile, int unit,
+                                           float* acc) {
+  for (; k0 < k1; k0 += kShortInFlight) {
+    int m[kShortInFlight];
+    uint4 r[kShortInFlight];
+#pragma unroll
+    for (int i = 0; i < kShortInFlight; ++i) m[i] = k0 + i < k1 ? __ldg(pt.map[k0 + i] + tile) : -1;
+#pragma unroll
+    for (int i = 0; i < kShortInFlight; ++i)
+      if (m[i] >= 0) r[i] = __ldcs(pt.data[k0 + i] + (size_t)m[i] * kPackedThreads + unit);
+#pragma unroll
+    for (int i = 0; i < kShortInFlight; ++i) {
+      if (m[i] < 0) continue;
+      float f[8];
+      unpack_h8(r[i], f);
+      fold<2>(acc, f);
+    }
+  }
+}
+
+// SHORT (sides of at most kShortLayers layers): 128 threads fold F, then B.  Otherwise F by the
+// first half of 256 threads and B by the second, each over the list of the layers that store the
+// tile.
+template <bool SHORT>
+__global__ void __launch_bounds__(SHORT ? kPackedThreads : 2 * kPackedThreads, SHORT ? kShortCtas : 1)
 composite_packed_kernel(const __grid_constant__ PackedTable pt, int nf, int nb, int width,
                         int height, int tiles_x, void* Fout, void* Bout, int out_f16) {
   pdl_prologue();
-  __shared__ int s_map[kMaxLayers], s_list[2][kMaxLayers], s_count[2];
   const int tile = blockIdx.x;
-  const int side = threadIdx.x / kPackedThreads;
   const int unit = threadIdx.x % kPackedThreads;      // pixels 2 unit, 2 unit + 1 of the tile
-  for (int k = threadIdx.x; k < nf + nb; k += blockDim.x) s_map[k] = __ldg(pt.map[k] + tile);
-  __syncthreads();
-  compact_stored(s_map, side ? nf : 0, side ? nf + nb : nf, unit, s_list[side], &s_count[side]);
-  __syncthreads();
-  void* out = side ? Bout : Fout;
-  if (!out) return;
   const int r = unit / (kTile / 2), c = 2 * (unit % (kTile / 2));
   const int y = (tile / tiles_x) * kTile + r, x = (tile % tiles_x) * kTile + c;
   float acc[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-  for_each_listed(pt.data, s_map, s_list[side], 0, s_count[side], unit, [&](int, uint4 v) {
-    float f[8];
-    unpack_h8(v, f);
-    fold<2>(acc, f);
-  });
-  if (y < height) {
+  auto put = [&](void* out) {
+    if (y >= height) return;
     if (x < width) store_pixel_out(out, out_f16, (long long)y * width + x, acc);
     if (x + 1 < width) store_pixel_out(out, out_f16, (long long)y * width + x + 1, acc + 4);
+  };
+  if (SHORT) {
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      void* out = side ? Bout : Fout;
+      if (!out) continue;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+      fold_short(pt, side ? nf : 0, side ? nf + nb : nf, tile, unit, acc);
+      put(out);
+    }
+  } else {
+    __shared__ int s_map[kMaxLayers], s_list[2][kMaxLayers], s_count[2];
+    const int side = threadIdx.x / kPackedThreads;
+    for (int k = threadIdx.x; k < nf + nb; k += blockDim.x) s_map[k] = __ldg(pt.map[k] + tile);
+    __syncthreads();
+    compact_stored(s_map, side ? nf : 0, side ? nf + nb : nf, unit, s_list[side], &s_count[side]);
+    __syncthreads();
+    void* out = side ? Bout : Fout;
+    if (!out) return;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+    for_each_listed(pt.data, s_map, s_list[side], 0, s_count[side], unit, [&](int, uint4 v) {
+      float f[8];
+      unpack_h8(v, f);
+      fold<2>(acc, f);
+    });
+    put(out);
   }
 }
 
@@ -421,10 +468,13 @@ extern "C" abcd_status abcd_composite_cache_packed(abcd_ctx* ctx, const int* con
     return fail(ctx, ABCD_ERR_INVALID_ARG, "abcd_composite_cache_packed: misaligned output");
   if (!F_out && !B_out) return ABCD_OK;
   const int tiles_x = (width + kTile - 1) / kTile, tiles_y = (height + kTile - 1) / kTile;
+  const int out_f16 = out_dtype == ABCD_F16 ? 1 : 0;
+  const bool few = std::max(nf, nb) <= kShortLayers;
   return check_launch(ctx, "composite_packed_kernel",
-                      launch_pdl(composite_packed_kernel, dim3(tiles_x * tiles_y),
-                                 dim3(2 * kPackedThreads), 0, ctx->stream, pt, nf, nb, width, height,
-                                 tiles_x, F_out, B_out, out_dtype == ABCD_F16 ? 1 : 0));
+                      launch_pdl(few ? composite_packed_kernel<true> : composite_packed_kernel<false>,
+                                 dim3(tiles_x * tiles_y),
+                                 dim3(few ? kPackedThreads : 2 * kPackedThreads), 0, ctx->stream, pt,
+                                 nf, nb, width, height, tiles_x, F_out, B_out, out_f16));
 }
 
 // ---- visibility of the layers of one camera's depth order (Section 4: visibility thresholds

@@ -649,6 +649,29 @@ def test_composite_packed_matches_dense(ctx):
             assert torch.equal(a_.view(torch.int16), b_.view(torch.int16)), split
 
 
+@pytest.mark.parametrize("nf,nb", [(0, 1), (4, 5), (8, 8), (8, 9), (9, 0), (33, 40)])
+def test_composite_packed_layer_counts(ctx, nf, nb):
+    """The packed composite with few layers per side (folded without a list) and with more, against
+    the dense one bit for bit; one layer stores nothing."""
+    H, W, L, split = 40, 72, nf + 1 + nb, nf
+    tx, ty = oracle.tiles_xy(W, H)
+    st = sg.premultiplied_layers(L, H, W, seed=23).astype(np.float16)
+    rng = np.random.default_rng(nf * 100 + nb)
+    for k in range(L):
+        for t in np.nonzero(rng.random(tx * ty) < (1.0 if k == L - 1 else 0.5))[0]:
+            st[k, (t // tx) * 16:(t // tx) * 16 + 16, (t % tx) * 16:(t % tx) * 16 + 16] = 0
+    enc = [pack_layer(st[k], tx, ty) for k in range(L)]
+    maps = [torch.from_numpy(m).cuda() for m, _ in enc]
+    packs = [torch.from_numpy(p if len(p) else np.zeros((1, 16, 16, 4), np.float16)).cuda() for _, p in enc]
+    dense = [torch.from_numpy(st[k]).cuda() for k in range(L)]
+    outs = [torch.empty(H, W, 4, dtype=torch.float16, device="cuda") for _ in range(4)]
+    ab.abcd_composite_cache(ctx, dense, list(range(L)), split, W, H, outs[0], outs[1])
+    ab.abcd_composite_cache_packed(ctx, maps, packs, list(range(L)), split, W, H, outs[2], outs[3])
+    ctx.sync()
+    for a_, b_ in zip(outs[:2], outs[2:]):
+        assert torch.equal(a_.view(torch.int16), b_.view(torch.int16))
+
+
 def _blank_tiles(st, tx, ty, share, seed):
     """Zero a random share of each layer's 16x16 tiles (the layers' transparent regions)."""
     rng = np.random.default_rng(seed)
