@@ -22,6 +22,7 @@ constexpr long long kMaxDiffCells = 1LL << 20;   // (tiles_x + 1) * (tiles_y + 1
 constexpr int kMaxRunRows = 1024;     // tile grids that bin through tile-row runs: rows ...
 constexpr int kMaxRunCols = 256;      // ... and columns at most
 constexpr int kVisSumCopies = 8;          // copies of the layer visibility sums
+constexpr int kSmemKernels = 16;          // kernels with dynamic shared memory, at most
 
 // Device status bits (OR-ed into the status word; abcd_sync reports the lowest set code).
 constexpr unsigned kStatusCapacity = 1u << ABCD_ERR_CAPACITY;
@@ -157,10 +158,9 @@ struct abcd_ctx {
   unsigned krange_parity = 0;           // which pair of depth-key range words bin_sort uses next
   unsigned wait_limit = 1u << 20;       // polls before a device-side wait gives up
   long long withhold_tile = -1;         // test hook: a look-back tile that publishes nothing
-  // dynamic shared memory limits already raised on this context's device, per kernel (the
-  // attribute call costs host time on every step otherwise)
-  const void* smem_fn[16] = {nullptr};
-  int smem_set[16] = {0};
+  // kernels whose dynamic shared memory limit this context has raised (the attribute calls cost
+  // host time on every step otherwise)
+  const void* smem_fn[abcd::kSmemKernels] = {nullptr};
   char err[512] = {0};
 };
 
@@ -170,8 +170,8 @@ abcd_status fail(abcd_ctx* ctx, abcd_status code, const char* fmt, ...);
 void cache_destroy(abcd_ctx* ctx);            // copy streams and slot events (cache.cu)
 abcd_status check_launch(abcd_ctx* ctx, const char* what);
 abcd_status check_launch(abcd_ctx* ctx, const char* what, cudaError_t launched);
-// Raises kernel fn's dynamic shared-memory limit to at least `bytes` (once per context and size).
-cudaError_t ensure_smem(abcd_ctx* ctx, const void* fn, size_t bytes);
+// Raises kernel fn's dynamic shared-memory limit to what the device offers (once per context).
+cudaError_t allow_smem(abcd_ctx* ctx, const void* fn);
 // Zeroes bytes at p on the context's stream with a programmatically serialised kernel (a memset
 // when p or bytes is not a multiple of 4).
 abcd_status zero_async(abcd_ctx* ctx, void* p, size_t bytes, const char* what);

@@ -1479,7 +1479,7 @@ abcd_status abcd::bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n, con
                             : 0;
     auto kern = by_runs ? tile_rows_kernel<true> : tile_rows_kernel<false>;
     {
-      const cudaError_t e2 = ensure_smem(ctx, (const void*)kern, smem);
+      const cudaError_t e2 = allow_smem(ctx, (const void*)kern);
       if (e2 != cudaSuccess) return fail(ctx, ABCD_ERR_CUDA, "tile_rows smem: %s", cudaGetErrorString(e2));
     }
     if ((s = check_launch(ctx, "tile_rows_kernel",
@@ -1495,7 +1495,7 @@ abcd_status abcd::bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n, con
     if (cells <= kSmemDiffCells && n_tiles <= ctx->ws.max_tiles) {
       const size_t smem = sizeof(int) * cells + (size_t)n_tiles;
       {
-        const cudaError_t e2 = ensure_smem(ctx, (const void*)ranges_order_kernel, smem);
+        const cudaError_t e2 = allow_smem(ctx, (const void*)ranges_order_kernel);
         if (e2 != cudaSuccess) return fail(ctx, ABCD_ERR_CUDA, "ranges smem: %s", cudaGetErrorString(e2));
       }
       if ((s = check_launch(ctx, "ranges_order_kernel",
@@ -1556,7 +1556,7 @@ abcd_status abcd::bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n, con
     const unsigned resident = (unsigned)ctx->num_sms *
                               (unsigned)std::max<size_t>(1, std::min<size_t>(8, (200u << 10) / (psm + 2048)));
     {
-      const cudaError_t e2 = ensure_smem(ctx, (const void*)place_kernel, psm);
+      const cudaError_t e2 = allow_smem(ctx, (const void*)place_kernel);
       if (e2 != cudaSuccess) return fail(ctx, ABCD_ERR_CUDA, "place smem: %s", cudaGetErrorString(e2));
     }
     return check_launch(ctx, "place_kernel",

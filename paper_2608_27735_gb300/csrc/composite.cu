@@ -656,7 +656,7 @@ abcd_status visibility_launch(abcd_ctx* ctx, const char* who, VisTable& vt, bool
   const size_t smem = own ? own_bytes : 0;
   const auto kernel = packed ? (own ? visibility_kernel<true, true> : visibility_kernel<true, false>)
                              : (own ? visibility_kernel<false, true> : visibility_kernel<false, false>);
-  const cudaError_t e = ensure_smem(ctx, (const void*)kernel, smem);
+  const cudaError_t e = allow_smem(ctx, (const void*)kernel);
   if (e != cudaSuccess) return fail(ctx, ABCD_ERR_CUDA, "%s smem: %s", who, cudaGetErrorString(e));
   return check_launch(ctx, "visibility_kernel",
                       launch_pdl(kernel, dim3(grid), dim3(kPackedThreads), smem, ctx->stream, vt,

@@ -65,20 +65,23 @@ abcd_status zero_async(abcd_ctx* ctx, void* p, size_t bytes, const char* what) {
                                             ctx->stream, (unsigned*)p, words));
 }
 
-cudaError_t ensure_smem(abcd_ctx* ctx, const void* fn, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  int slot = -1;
-  for (int i = 0; i < 16; ++i) {
-    if (ctx->smem_fn[i] == fn) { slot = i; break; }
-    if (!ctx->smem_fn[i] && slot < 0) slot = i;
-  }
-  if (slot >= 0 && ctx->smem_fn[slot] == fn && ctx->smem_set[slot] >= (int)bytes) return cudaSuccess;
-  int prev = 0;
+// A launch needs the opt-in when its static and dynamic shared memory together exceed 48 KB, whatever
+// the dynamic size alone is.  The limit is one per kernel and device, shared by every context: each
+// sets it to all that the device offers, so none lowers another's.
+cudaError_t allow_smem(abcd_ctx* ctx, const void* fn) {
+  int slot = 0;
+  while (slot < kSmemKernels && ctx->smem_fn[slot] && ctx->smem_fn[slot] != fn) ++slot;
+  if (slot < kSmemKernels && ctx->smem_fn[slot] == fn) return cudaSuccess;
+  int prev = 0, optin = 0;
+  cudaFuncAttributes at = {};
   cudaGetDevice(&prev);
   if (prev != ctx->device) cudaSetDevice(ctx->device);
-  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaError_t e = cudaFuncGetAttributes(&at, fn);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)at.sharedSizeBytes);
   if (prev != ctx->device) cudaSetDevice(prev);
-  if (e == cudaSuccess && slot >= 0) { ctx->smem_fn[slot] = fn; ctx->smem_set[slot] = (int)bytes; }
+  if (e == cudaSuccess && slot < kSmemKernels) ctx->smem_fn[slot] = fn;
   return e;
 }
 

@@ -668,8 +668,8 @@ abcd_status loss_launch(abcd_ctx* ctx, const float* out_rgba, const float* gt_rg
   if ((long long)grid.x * grid.y * grid.z > kMaxLossBlocks)
     return fail(ctx, ABCD_ERR_INVALID_ARG, "abcd_loss: image too large (%d x %d)", width, height);
   const size_t smem_f = sizeof(float) * kQFwdFloats, smem_b = sizeof(float) * kQBwdFloats;
-  cudaError_t e = ensure_smem(ctx, (const void*)ssim_fwd_kernel, smem_f);
-  if (e == cudaSuccess && dL_dout) e = ensure_smem(ctx, (const void*)ssim_bwd_kernel, smem_b);
+  cudaError_t e = allow_smem(ctx, (const void*)ssim_fwd_kernel);
+  if (e == cudaSuccess && dL_dout) e = allow_smem(ctx, (const void*)ssim_bwd_kernel);
   if (e != cudaSuccess) return fail(ctx, ABCD_ERR_CUDA, "loss smem attribute: %s", cudaGetErrorString(e));
   const Window win = ssim_window();
   float2* abc_ab = dL_dout ? ctx->ws.ssim_ab : nullptr;

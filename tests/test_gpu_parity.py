@@ -234,6 +234,24 @@ def test_bin_sort_wide_image(ctx, W, H):
     print(f"{W}x{H}: K = {K}, optional entries {n_opt} ({share:.2e} of K)")
 
 
+@pytest.mark.parametrize("W,H", [(1920, 1120), (1920, 1160), (1920, 1280), (1920, 1296)])
+def test_bin_sort_shared_memory_limit(ctx, W, H):
+    """Tile grids whose cells, tile keys and the range kernel's own arrays fit in 48 KB of shared
+    memory together (8,400 tiles), or only the cells and keys by themselves (8,760 and 9,600), or
+    not at all (9,720)."""
+    s = sg.grid_scene((1, 1, 1), 5.0, 500, 0, seed=96)
+    s.cameras = sg.ring_cameras(1, 1.5 * sg.half_diagonal(s.grid), np.zeros(3), W, H, seed=96,
+                                height_jitter=1.0)
+    ctx.reserve(500, 2_000_000, W * H)
+    case = Case(s, 0, fb=False)
+    r = run_forward(ctx, case, want_state=False)
+    K = int(r["tiles"].count.item())
+    rng = r["tiles"].ranges.cpu().numpy().astype(np.int64)
+    ids = r["tiles"].ids.cpu().numpy()[:K]
+    tx, ty = oracle.tiles_xy(case.cam.width, case.cam.height)
+    par.check_tile_lists(rng, ids, case.off, case.ids, case.P, case.opt_list, tx * ty)
+
+
 @pytest.mark.parametrize("cam_idx,bg,fbdt", [(0, None, "f16"), (1, (0.2, 0.5, 0.9), "f16"),
                                              (2, None, "f32"), (3, (1.0, 1.0, 1.0), "f16")])
 def test_render_composite_fwd_matches_oracle(ctx, tiny, cam_idx, bg, fbdt):
@@ -721,6 +739,28 @@ def test_layer_visibility_matches_oracle(ctx, H, W, L):
         np.testing.assert_allclose(got[0][1], cr, rtol=0, atol=tol)
         for g in got[1:]:
             assert np.array_equal(g[0], got[0][0]) and np.array_equal(g[1], got[0][1])
+
+
+@pytest.mark.parametrize("L", [41, 42, 45, 48, 49])
+def test_layer_visibility_shared_memory_limit(ctx, L):
+    """Layer counts whose sums and the kernel's own arrays fit in 48 KB of shared memory together,
+    or only each by itself, or not at all."""
+    H, W = 40, 56
+    tx, ty = oracle.tiles_xy(W, H)
+    st = _blank_tiles(sg.premultiplied_layers(L, H, W, seed=90 + L).astype(np.float16), tx, ty, 0.3, 7)
+    enc = [pack_layer(st[k], tx, ty) for k in range(L)]
+    maps = [torch.from_numpy(m).cuda() for m, _ in enc]
+    packs = [torch.from_numpy(p if len(p) else np.zeros((1, 16, 16, 4), np.float16)).cuda() for _, p in enc]
+    dense = [torch.from_numpy(st[k]).cuda() for k in range(L)]
+    order = list(sg.random_permutation(L, seed=L))
+    vr, cr = oracle.layer_visibility(st.astype(np.float64), order)
+    got = [torch.empty(L, dtype=torch.float64, device="cuda") for _ in range(4)]
+    ab.abcd_layer_visibility(ctx, dense, order, W, H, got[0], got[1])
+    ab.abcd_layer_visibility_packed(ctx, maps, packs, order, W, H, got[2], got[3])
+    ctx.sync()
+    for g, ref in zip(got, (vr, cr, vr, cr)):
+        np.testing.assert_allclose(g.cpu().numpy(), ref, rtol=0, atol=visibility_tol(L))
+    assert torch.equal(got[0], got[2]) and torch.equal(got[1], got[3])
 
 
 def test_layer_visibility_occlusion_and_errors(ctx):
