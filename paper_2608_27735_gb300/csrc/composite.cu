@@ -5,11 +5,16 @@
 //
 // Pure streaming work: every layer is read once (16-byte streaming loads, evict-first), the
 // accumulator stays in registers across layers, F and B are written once.  Four layers are
-// loaded before they are folded so each thread keeps 64 bytes in flight, the last one to three
-// of a side together too (64 layers at 1080p 185 -> 181 us, 5.9 TB/s; 27 layers at 640x480 with
-// their loss 31.4 -> 28.7 us).  Eight in flight take 97 registers and are slower (215 us); one
-// pixel per thread on small images is, too (30.7 us).  The grid is a multiple of the SM count
-// and strides over pixel pairs.
+// loaded before they are folded, the last one to three of a side together too.  What bounds it is
+// the loads an SM has in flight, so the CTAs on an SM count as much as the loads of a thread: fp16
+// layers and single pixels keep to 32 registers, eight CTAs, so the grid of eight per SM (which
+// strides over the pixel pairs) is resident at once; pairs of 32-bit layers take 40, six CTAs.
+// 64 fp16 layers at 1080p take 154 us (6.8 TB/s), 27 at 1236x822 31.8, at 864x600 15.4, at 640x480
+// 14.2 (bound by the host); 33 32-bit layers at 1080p 159.5, 27 at 1236x822 65.7.  At seven CTAs
+// (36 registers) the fp16 figures are 182, 40.5, 24.8 and 14.0; with a predicated tail of four
+// loads (58 registers, pairs of 32-bit layers 86) 174, 41.9, 20.4 and 14.0, and the 32-bit ones 239
+// and 97.  Eight layers in flight are slower (215 us at 1080p), one pixel per thread on small
+// images too.
 #include <algorithm>
 
 #include "abcd_internal.cuh"
@@ -79,36 +84,29 @@ struct Raw {
   }
 };
 
-constexpr int kInFlight = 4;
+// acc = acc over layers [k, k + N), their loads in flight together.
+template <int N, int PIX, bool F16>
+__device__ __forceinline__ void fold_n(const LayerTable& lt, int k, long long g, float* acc) {
+  Raw<PIX, F16> v[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) v[j].load(lt.p[k + j], g);
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    float f[4 * PIX];
+    v[j].unpack(f);
+    fold<PIX>(acc, f);
+  }
+}
 
 template <int PIX, bool F16>
 __device__ __forceinline__ void fold_range(const LayerTable& lt, int k0, int k1, long long g,
                                            float* acc) {
   int k = k0;
-  for (; k + kInFlight <= k1; k += kInFlight) {
-    Raw<PIX, F16> v[kInFlight];
-#pragma unroll
-    for (int j = 0; j < kInFlight; ++j) v[j].load(lt.p[k + j], g);
-#pragma unroll
-    for (int j = 0; j < kInFlight; ++j) {
-      float f[4 * PIX];
-      v[j].unpack(f);
-      fold<PIX>(acc, f);
-    }
-  }
-  if (k < k1) {                                      // the rest, also in flight together
-    Raw<PIX, F16> v[kInFlight];
-#pragma unroll
-    for (int j = 0; j < kInFlight; ++j)
-      if (k + j < k1) v[j].load(lt.p[k + j], g);
-#pragma unroll
-    for (int j = 0; j < kInFlight; ++j) {
-      if (k + j >= k1) break;
-      float f[4 * PIX];
-      v[j].unpack(f);
-      fold<PIX>(acc, f);
-    }
-  }
+  for (; k + 4 <= k1; k += 4) fold_n<4, PIX, F16>(lt, k, g, acc);
+  const int rest = k1 - k;
+  if (rest == 3) fold_n<3, PIX, F16>(lt, k, g, acc);
+  else if (rest == 2) fold_n<2, PIX, F16>(lt, k, g, acc);
+  else if (rest == 1) fold_n<1, PIX, F16>(lt, k, g, acc);
 }
 
 template <int PIX>
@@ -131,8 +129,9 @@ __device__ __forceinline__ void store_group(void* out, int f16, long long g, con
   }
 }
 
+// (0 CTAs: left to the compiler, which takes 40 registers; six asked for cost it two spills)
 template <int PIX, bool F16>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, PIX == 1 || F16 ? 8 : 0)
 composite_kernel(const __grid_constant__ LayerTable lt, int nf, int nb, long long groups,
                  void* Fout, void* Bout, int out_f16) {
   pdl_wait();

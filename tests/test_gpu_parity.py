@@ -529,6 +529,25 @@ def test_composite_cache_matches_oracle(ctx, dtype, out_dtype, H, W, L):
                 assert exact.mean() > 0.99
 
 
+@pytest.mark.parametrize("dtype", ["f16", "f32"])
+@pytest.mark.parametrize("H,W", [(19, 27), (18, 26)])
+@pytest.mark.parametrize("nf,nb", [(0, 1), (1, 2), (2, 3), (3, 4), (4, 5), (6, 7)])
+def test_composite_cache_remainders(ctx, dtype, H, W, nf, nb):
+    """Every remainder of four layers on either side, single pixels (an odd image) and pairs."""
+    L = nf + 1 + nb
+    st = sg.premultiplied_layers(L, H, W, seed=10 * nf + nb).astype(np.float16 if dtype == "f16" else np.float32)
+    layers = [torch.from_numpy(st[k]).cuda() for k in range(L)]
+    F, B = (torch.empty(H, W, 4, device="cuda") for _ in range(2))
+    ab.abcd_composite_cache(ctx, layers, list(range(L)), nf, W, H, F, B,
+                            ab.ABCD_F16 if dtype == "f16" else ab.ABCD_F32, ab.ABCD_F32)
+    ctx.sync()
+    src = st.astype(np.float64)
+    for got, order in ((F, range(nf)), (B, range(nf + 1, L))):
+        ref = oracle.composite_layers(src, list(order)) if len(order) else np.zeros((H, W, 4))
+        # one fused multiply-add per layer and 1 - a, each rounded once, on values in [0, 1]
+        assert np.abs(got.cpu().numpy() - ref).max() <= 2 * L * 2.0 ** -24
+
+
 def check_fb16(got, ref, L):
     """fp16 composite output against the exact fold (fp32 accumulation, one rounding)."""
     g = got.cpu().numpy()
