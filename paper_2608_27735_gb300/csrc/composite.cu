@@ -494,11 +494,16 @@ namespace {
 
 constexpr float kVisScale = 16777216.f;       // 2^24
 constexpr int kVisInFlight = 8;               // layers whose loads are in flight together
-// Positions with sums per thread: 64 take 64 KB per CTA and leave two on an SM, above that the
-// CTA's sums cost less.  32 layers at 1237x822, a third of the tiles stored: 26 us against 31 us
-// with a warp reduction and a shared atomic per layer, tile and sum (both bound by latency: 3.4
-// of 6.8 TB/s).
-constexpr int kVisOwnLayers = 64;
+// Most positions with sums per thread.  A position takes 1 KB of a CTA's shared memory, and what that
+// leaves bounds the rest: packed layers, streamed past the L1, need the five CTAs that 32 positions
+// allow on an SM; dense ones, of which the two loads of a pixel pair share cache lines, need the L1
+// that eight CTAs of 14 leave.  Above, a warp reduction and a shared atomic per layer, tile and sum
+// (both forms are bound by latency: 3.4 of 6.8 TB/s).  At 1237x822 (us, sums per thread / reduction):
+// packed, 0.4 of the tiles stored, 20 layers 17 / 23, 32: 27 / 32, 33: 33 / 33, 64: 87 / 53; at 1080p,
+// a tenth stored, 32: 22 / 28, 33: 34 / 30.  Dense 12 layers 23 / 29, 14: 26 / 32, 16: 44 / 35,
+// 32: 85 / 61.
+constexpr int kVisOwnPacked = 32;
+constexpr int kVisOwnDense = 14;
 constexpr int kVisCopies = kVisSumCopies;     // global accumulators (CTA b adds to copy b % 8)
 
 struct VisTable {
@@ -646,11 +651,12 @@ abcd_status visibility_launch(abcd_ctx* ctx, const char* who, VisTable& vt, bool
     return fail(ctx, ABCD_ERR_INVALID_ARG, "%s: null or misaligned output", who);
   const int tiles_x = (width + kTile - 1) / kTile, tiles_y = (height + kTile - 1) / kTile;
   const int n_tiles = tiles_x * tiles_y;
-  // per-thread sums while they fit in shared memory with enough CTAs on an SM, and cannot
+  // per-thread sums while they leave enough CTAs and L1 (kVisOwnPacked, kVisOwnDense), and cannot
   // overflow: a tile adds at most 2^25 to a 32-bit sum
   const size_t own_bytes = sizeof(uint2) * kPackedThreads * (size_t)count;
   const int own_ctas = std::max(1, std::min<int>(8, (int)((200u << 10) / (own_bytes + (8u << 10)))));
-  const bool own = count <= kVisOwnLayers && n_tiles <= 64LL * own_ctas * ctx->num_sms;
+  const bool own = count <= (packed ? kVisOwnPacked : kVisOwnDense) &&
+                   n_tiles <= 64LL * own_ctas * ctx->num_sms;
   const int grid = std::max(1, std::min(n_tiles, (own ? own_ctas : 8) * ctx->num_sms));
   const size_t smem = own ? own_bytes : 0;
   const auto kernel = packed ? (own ? visibility_kernel<true, true> : visibility_kernel<true, false>)

@@ -782,6 +782,72 @@ def test_layer_visibility_shared_memory_limit(ctx, L):
     assert torch.equal(got[0], got[2]) and torch.equal(got[1], got[3])
 
 
+@pytest.mark.parametrize("L", [14, 15, 32, 33, 64, 65, 130])
+def test_layer_visibility_forms(ctx, L):
+    """Sums kept by each thread (up to 14 dense layers, 32 packed ones) and reduced per warp: the
+    integers are the same, so dense and packed calls give the same bits on either side of both."""
+    H, W = 37, 45
+    tx, ty = oracle.tiles_xy(W, H)
+    st = _blank_tiles(sg.premultiplied_layers(L, H, W, seed=60 + L).astype(np.float16), tx, ty, 0.4, 8)
+    enc = [pack_layer(st[k], tx, ty) for k in range(L)]
+    maps = [torch.from_numpy(m).cuda() for m, _ in enc]
+    packs = [torch.from_numpy(p if len(p) else np.zeros((1, 16, 16, 4), np.float16)).cuda() for _, p in enc]
+    dense = [torch.from_numpy(st[k]).cuda() for k in range(L)]
+    order = list(sg.random_permutation(L, seed=L))
+    vr, cr = oracle.layer_visibility(st.astype(np.float64), order)
+    got = [torch.empty(L, dtype=torch.float64, device="cuda") for _ in range(4)]
+    ab.abcd_layer_visibility(ctx, dense, order, W, H, got[0], got[1])
+    ab.abcd_layer_visibility_packed(ctx, maps, packs, order, W, H, got[2], got[3])
+    ctx.sync()
+    for g, ref in zip(got, (vr, cr, vr, cr)):
+        np.testing.assert_allclose(g.cpu().numpy(), ref, rtol=0, atol=visibility_tol(L))
+    assert torch.equal(got[0], got[2]) and torch.equal(got[1], got[3])
+
+
+@pytest.mark.parametrize("rows_over", [0, 1])
+def test_layer_visibility_tile_limit(ctx, rows_over):
+    """The most tiles whose sums a thread keeps in 32 bits (64 tiles of two opaque pixels: 2^31) and
+    one tile row more: an opaque layer is visible and covered everywhere, exactly."""
+    W = 4096
+    H = 16 * (64 * 8 * torch.cuda.get_device_properties(0).multi_processor_count // (W // 16) + rows_over)
+    layer = torch.ones(H, W, 4, dtype=torch.float16, device="cuda")
+    vis, cov = (torch.zeros(1, dtype=torch.float64, device="cuda") for _ in range(2))
+    ab.abcd_layer_visibility(ctx, [layer], [0], W, H, vis, cov)
+    ctx.sync()
+    assert vis.item() == 1.0 and cov.item() == 1.0
+
+
+@pytest.mark.parametrize("packed,few,many,most", [(True, 32, 64, 2.6), (False, 14, 32, 2.8)])
+def test_layer_visibility_cost_of_more_layers(ctx, packed, few, many, most):
+    """The sums per thread end where they crowd out what hides the loads' latency: 64 packed layers
+    take twice as long as 32 and 32 dense ones 2.35 times as long as 14 (3.2 and 3.3 times, kept in
+    shared memory all the same)."""
+    H, W = 822, 1237
+    tx, ty = oracle.tiles_xy(W, H)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    vis, cov = (torch.zeros(many, dtype=torch.float64, device="cuda") for _ in range(2))
+    if packed:
+        stored = [torch.rand(tx * ty, generator=g, device="cuda") < 0.4 for _ in range(many)]
+        maps = [torch.where(s, s.int().cumsum(0, dtype=torch.int32) - 1, -1).int().contiguous() for s in stored]
+        data = [torch.rand(int(s.sum()), 16, 16, 4, generator=g, device="cuda").half() for s in stored]
+        call = lambda n: ab.abcd_layer_visibility_packed(ctx, maps[:n], data[:n], list(range(n)), W, H, vis[:n], cov[:n])
+    else:
+        layers = [torch.rand(H, W, 4, generator=g, device="cuda").half() for _ in range(many)]
+        call = lambda n: ab.abcd_layer_visibility(ctx, layers[:n], list(range(n)), W, H, vis[:n], cov[:n])
+    best = {}
+    for n in (few, many, few, many):
+        for _ in range(12):
+            torch.cuda._sleep(400_000)               # the calls queue up: host time does not count
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(4):
+                call(n)
+            b.record()
+            ctx.sync()
+            best[n] = min(best.get(n, 1e9), a.elapsed_time(b))
+    assert best[many] <= most * best[few], best
+
+
 def test_layer_visibility_occlusion_and_errors(ctx):
     """An opaque layer in front hides every layer behind it exactly; coverage ignores it; a
     culled composite stays within the bound the dropped layers' visible shares give; bad
