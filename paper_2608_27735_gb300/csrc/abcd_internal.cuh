@@ -91,8 +91,7 @@ constexpr int kRenderSubPerTile = 4;      // render CTAs (8x8 pixel blocks) per 
 // some SMs and few on others, in launch order (the longest render walks next to each other), and
 // holding slots meanwhile.  That pays only where this grid is short and the next one's CTAs are
 // few and alike: project_fwd -> keys_rects -> sort_digits -> the first radix pass, zero_kernel (a
-// short kernel ahead of the render kernels), composite_packed_kernel (19.6 against 19.8 us), and
-// the one-CTA and whole-loss kernels outside the step.
+// short kernel ahead of the render kernels), and the one-CTA and whole-loss kernels outside the step.
 //
 // The step with every trigger early, every one late, and as built (us): 2,000 Gaussians at 128x128
 // 103 / 96 / 96; 20,000 at 640x480 171 / 160 / 160; 33,000 at 1001x667 243 / 242 / 239; 100,000 at

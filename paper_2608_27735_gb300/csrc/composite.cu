@@ -203,13 +203,9 @@ extern "C" abcd_status abcd_composite_cache(abcd_ctx* ctx, const void* const* la
 }
 
 // ---- K1 over packed layers (the cache's tile-sparse format, see abcd_render_refresh_packed):
-// one CTA per 16x16 tile, two pixels per thread, the tile's map entries of all layers read
-// once into shared memory and compacted into the list of those that store it, so that all eight
-// loads a thread has in flight are real (32 layers at 1237x822, a third stored, F and B by two
-// halves of the CTA side by side: 21.4 -> 19.5 us, 5.2 TB/s; what is left is the latency of map,
-// list and loads per tile); a layer whose tile is not stored is transparent, and folding
-// (0, 0, 0, 0) leaves the accumulator unchanged, so skipping it gives the dense result bit for
-// bit.  Only the stored tiles are read.
+// one CTA per 16x16 tile, two pixels per thread; a layer whose tile is not stored is transparent,
+// and folding (0, 0, 0, 0) leaves the accumulator unchanged, so skipping it gives the dense result
+// bit for bit.  Only the stored tiles are read.
 namespace abcd {
 namespace {
 
@@ -220,13 +216,23 @@ struct PackedTable {
 
 constexpr int kPackedThreads = kTileThreads / 2;
 constexpr int kPackedInFlight = 8;
-// Sides of up to kShortLayers layers are folded without the list (F, then B, by 128 threads, no
-// shared memory): with few layers its barriers cost more than its loads gain.  At 1210x883, a
-// tenth and nine tenths of the tiles stored: 3 layers 9.4 -> 6.9 and 12.6 -> 8.7 us; 9 layers 10.2
-// -> 8.7, half stored 14.6 -> 11.5; 13 layers, a third stored, 14.3 -> 12.3.  Without the line 24
-// layers take 18.6 against 17.0 us and 64 (a tenth stored) 33 against 19.  Four loads in flight
-// and 12 CTAs per SM (40 registers): eight take 8.2 us for 3 layers, 16 CTAs spill.
-constexpr int kShortLayers = 8;
+// What bounds the composite is latency -- the tile's map entries, then its layers -- against the
+// CTAs that hide it.  Two warps list the layers that store the tile, one per side, so that all eight
+// loads a thread has in flight are real; 56 registers keep nine CTAs on an SM.  32 layers at 1237x822
+// (16 front, 15 back), 0.1 / 0.4 / 0.9 of the tiles stored: 8.4 / 18.1 / 34.7 us (0.4: 6.6 TB/s) against
+// 12.6 / 23.2 / 41.6 without the list (eight layers at a time, the unstored ones masked, eight CTAs).
+// F and B by two halves of a 256-thread CTA took 11.6 / 21.1 / 36.2 and left half the CTA idle when
+// one side is empty: 16 front layers at 1080p, a tenth stored, 17.7 us against 12.3 here and 15.6
+// without the list.  The list as packed words or as addresses is no better; the next grid launched
+// early is worse (640x480, 16 and 16 layers, 0.9 stored: 9.3 against 8.7 us).
+constexpr int kListCtas = 9;
+// Sides of up to kShortLayers layers are folded without the list (F, then B, no shared memory): one
+// round of loads of the tile's map entries, one of its layers.  Against the list at 1080p, 0.4 / 0.9
+// of the tiles stored: 1 and 1 layers 11.1 / 12.5 against 12.1 / 16.3 us, 4 and 4 15.0 / 22.1 against
+// 16.7 / 24.0.  With 5 and 5 a second round of both follows: 15.8 us against 11.8 (a tenth stored).
+// Four loads in flight and 12 CTAs per SM (40 registers): eight take 8.2 against 6.9 us for 3 layers,
+// 16 CTAs spill.
+constexpr int kShortLayers = 4;
 constexpr int kShortInFlight = 4;
 constexpr int kShortCtas = 12;
 
@@ -312,51 +318,86 @@ __device__ __forceinline__ void fold_short(const PackedTable& pt, int k0, int k1
   }
 }
 
-// SHORT (sides of at most kShortLayers layers): 128 threads fold F, then B.  Otherwise F by the
-// first half of 256 threads and B by the second, each over the list of the layers that store the
-// tile.
+// A layer that stores the tile: its position in the table and the tile's block.
+struct Stored {
+  int layer, block;
+};
+
+// The layers of [k0, k1) that store the tile, in order, into list (one warp); returns how many.
+__device__ __forceinline__ int list_stored(const PackedTable& pt, int k0, int k1, int tile, Stored* list) {
+  constexpr int kMaps = 4;                             // map entries a lane has in flight
+  const int lane = threadIdx.x & 31;
+  int run = 0;
+  for (int b = k0; b < k1; b += 32 * kMaps) {
+    int m[kMaps];
+#pragma unroll
+    for (int i = 0; i < kMaps; ++i) {
+      const int k = b + 32 * i + lane;
+      m[i] = k < k1 ? __ldg(pt.map[k] + tile) : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < kMaps; ++i) {
+      const unsigned st = __ballot_sync(0xffffffffu, m[i] >= 0);
+      if (m[i] >= 0) list[run + __popc(st & ((1u << lane) - 1u))] = {b + 32 * i + lane, m[i]};
+      run += __popc(st);
+    }
+  }
+  return run;
+}
+
+// acc (2 pixels) = acc over the listed layers [j, j1), the loads of kPackedInFlight in flight together.
+__device__ __forceinline__ void fold_listed(const PackedTable& pt, const Stored* list, int j, int j1,
+                                            int unit, float* acc) {
+  for (; j < j1; j += kPackedInFlight) {
+    uint4 r[kPackedInFlight];
+#pragma unroll
+    for (int i = 0; i < kPackedInFlight; ++i) {
+      if (j + i >= j1) continue;
+      const Stored e = list[j + i];
+      r[i] = __ldcs(pt.data[e.layer] + (size_t)e.block * kPackedThreads + unit);
+    }
+#pragma unroll
+    for (int i = 0; i < kPackedInFlight; ++i) {
+      if (j + i >= j1) break;
+      float f[8];
+      unpack_h8(r[i], f);
+      fold<2>(acc, f);
+    }
+  }
+}
+
+// F, then B, by 128 threads; SHORT: sides of at most kShortLayers layers.
 template <bool SHORT>
-__global__ void __launch_bounds__(SHORT ? kPackedThreads : 2 * kPackedThreads, SHORT ? kShortCtas : 1)
+__global__ void __launch_bounds__(kPackedThreads, SHORT ? kShortCtas : kListCtas)
 composite_packed_kernel(const __grid_constant__ PackedTable pt, int nf, int nb, int width,
                         int height, int tiles_x, void* Fout, void* Bout, int out_f16) {
-  pdl_prologue();
+  pdl_wait();
+  __shared__ Stored s_list[SHORT ? 1 : kMaxLayers];
+  __shared__ int s_end[2];
   const int tile = blockIdx.x;
-  const int unit = threadIdx.x % kPackedThreads;      // pixels 2 unit, 2 unit + 1 of the tile
+  const int unit = threadIdx.x;                       // pixels 2 unit, 2 unit + 1 of the tile
   const int r = unit / (kTile / 2), c = 2 * (unit % (kTile / 2));
   const int y = (tile / tiles_x) * kTile + r, x = (tile % tiles_x) * kTile + c;
-  float acc[8];
-  auto put = [&](void* out) {
-    if (y >= height) return;
-    if (x < width) store_pixel_out(out, out_f16, (long long)y * width + x, acc);
-    if (x + 1 < width) store_pixel_out(out, out_f16, (long long)y * width + x + 1, acc + 4);
-  };
-  if (SHORT) {
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      void* out = side ? Bout : Fout;
-      if (!out) continue;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-      fold_short(pt, side ? nf : 0, side ? nf + nb : nf, tile, unit, acc);
-      put(out);
+  if (!SHORT) {
+    if (unit < 64) {
+      const int side = unit >> 5, k0 = side ? nf : 0, k1 = side ? nf + nb : nf;
+      const int n = list_stored(pt, k0, k1, tile, s_list + k0);
+      if ((unit & 31) == 0) s_end[side] = k0 + n;
     }
-  } else {
-    __shared__ int s_map[kMaxLayers], s_list[2][kMaxLayers], s_count[2];
-    const int side = threadIdx.x / kPackedThreads;
-    for (int k = threadIdx.x; k < nf + nb; k += blockDim.x) s_map[k] = __ldg(pt.map[k] + tile);
     __syncthreads();
-    compact_stored(s_map, side ? nf : 0, side ? nf + nb : nf, unit, s_list[side], &s_count[side]);
-    __syncthreads();
+  }
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
     void* out = side ? Bout : Fout;
-    if (!out) return;
+    if (!out) continue;
+    float acc[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-    for_each_listed(pt.data, s_map, s_list[side], 0, s_count[side], unit, [&](int, uint4 v) {
-      float f[8];
-      unpack_h8(v, f);
-      fold<2>(acc, f);
-    });
-    put(out);
+    if (SHORT) fold_short(pt, side ? nf : 0, side ? nf + nb : nf, tile, unit, acc);
+    else fold_listed(pt, s_list, side ? nf : 0, s_end[side], unit, acc);
+    if (y >= height) continue;
+    if (x < width) store_pixel_out(out, out_f16, (long long)y * width + x, acc);
+    if (x + 1 < width) store_pixel_out(out, out_f16, (long long)y * width + x + 1, acc + 4);
   }
 }
 
@@ -471,8 +512,7 @@ extern "C" abcd_status abcd_composite_cache_packed(abcd_ctx* ctx, const int* con
   const bool few = std::max(nf, nb) <= kShortLayers;
   return check_launch(ctx, "composite_packed_kernel",
                       launch_pdl(few ? composite_packed_kernel<true> : composite_packed_kernel<false>,
-                                 dim3(tiles_x * tiles_y),
-                                 dim3(few ? kPackedThreads : 2 * kPackedThreads), 0, ctx->stream, pt,
+                                 dim3(tiles_x * tiles_y), dim3(kPackedThreads), 0, ctx->stream, pt,
                                  nf, nb, width, height, tiles_x, F_out, B_out, out_f16));
 }
 
