@@ -38,7 +38,9 @@ struct Cam {               // camera as the kernels read it (by value)
 
 struct Opts {
   float near_z, dilation, alpha_max, alpha_min, t_min, guard;
-  float inv_alpha_min;     // 1 / alpha_min; inf when alpha_min <= 0: no entry is too faint
+  // 1 / alpha_min; the least limit of sigma (0, or inf when alpha_min <= 0: no entry is too faint);
+  // the opacity from which the limit needs no second look (4 alpha_min; none does without alpha_min)
+  float inv_alpha_min, least_limit, faint;
 };
 
 struct SHConst { float k[16]; };    // normalisation factors of the real SH basis

@@ -94,6 +94,8 @@ Opts make_opts(const abcd_render_opts* o) {
   r.alpha_min = o ? o->alpha_min : 1.0f / 255.0f;
   r.t_min = o ? o->t_min : 1e-4f;
   r.inv_alpha_min = r.alpha_min > 0.f ? 1.f / r.alpha_min : INFINITY;
+  r.least_limit = r.alpha_min > 0.f ? 0.f : INFINITY;
+  r.faint = r.alpha_min > 0.f ? 4.f * r.alpha_min : -INFINITY;
   return r;
 }
 

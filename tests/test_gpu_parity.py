@@ -389,6 +389,89 @@ def test_render_indefinite_conic_is_walked(ctx):
     assert bool((grad2d[2] == 0).all())
 
 
+def one_entry_per_tile(W, H, uv, conic_opacity):
+    """Projection and lists in which tile t lists Gaussian t alone, of colour 1."""
+    n = uv.shape[0]
+    proj = ab.Projected.alloc(n)
+    proj.uv.copy_(uv)
+    proj.conic_opacity.copy_(conic_opacity)
+    proj.rgb.fill_(1.0)
+    tiles = ab.Tiles.alloc(n, W, H)
+    tiles.ids.copy_(torch.arange(n, dtype=torch.int32))
+    tiles.ranges.copy_(torch.stack([torch.arange(n), torch.arange(n) + 1], 1).int())
+    return proj, tiles
+
+
+@pytest.mark.parametrize("lo,hi", [(1.0, 1.0 + 1e-5), (1.0, 1.01), (1.01, 1.2), (1.2, 1.5), (1.5, 2.3), (2.3, 250.0)])
+def test_render_limit_decides_as_the_alpha(ctx, lo, hi):
+    """Entries whose alpha is within a few units of its last place of alpha_min at a column of their
+    tile: a pixel takes them exactly where the alpha itself (the colour that the same entry leaves when
+    nothing is too faint) is at least alpha_min, and the backward decides alike."""
+    W = H = 1024
+    n, am = (W // 16) * (H // 16), np.float32(1.0 / 255.0)
+    rng = np.random.default_rng(int(1000 * hi))
+    o = (am * np.exp(rng.uniform(np.log(lo), np.log(hi), n))).astype(np.float32)
+    o = np.maximum(o, am)
+    # sigma log2(e) = a' dx^2 with dx = 1 .. 16 along a row, near its limit at dx = 9; the rows differ
+    # by a few 1e-8 through c
+    target = np.maximum(np.log2(o.astype(np.float64) / am) + rng.uniform(-6e-7, 6e-7, n), 0.0)
+    k = 0.5 * np.log2(np.e)
+    co = np.stack([target / 81.0 / k, np.zeros(n), rng.uniform(0.0, 4e-9, n) / k, o], 1).astype(np.float32)
+    t = np.arange(n)
+    uv = np.stack([16.0 * (t % (W // 16)) - 0.5, 16.0 * (t // (W // 16)) - 0.5], 1).astype(np.float32)
+    proj, tiles = one_entry_per_tile(W, H, torch.from_numpy(uv), torch.from_numpy(co))
+    cam = ab.camera(sg.look_at((0.0, -5.0, 0.0), np.zeros(3), W, H))
+    out, st = torch.empty(H, W, 4, device="cuda"), ab.FwdState.alloc(W, H)
+    got = []
+    for alpha_min in (0.0, float(am)):
+        opts = ab.render_opts(alpha_min=alpha_min)
+        ab.abcd_render_composite_fwd(ctx, cam, opts, proj, tiles, None, None, ab.ABCD_F16, None, out, st)
+        ctx.sync()
+        got.append((st.A_T[..., 0].clone(), st.n_last.clone()))
+    alpha = got[0][0]
+    assert bool((got[0][1] == 1).all())
+    taken = alpha >= torch.tensor(am, device="cuda")
+    near = (alpha - float(am)).abs() < 4e-7 * float(am)
+    assert int((near & taken).sum()) > 1000 and int((near & ~taken).sum()) > 1000
+    assert torch.equal(got[1][1] == 1, taken)
+    assert torch.equal(got[1][0], torch.where(taken, alpha, torch.zeros_like(alpha)))
+    grad2d = torch.empty(n, 9, device="cuda")
+    ab.abcd_render_backward(ctx, cam, opts, proj, tiles, None, None, ab.ABCD_F16, None, st,
+                            torch.ones(H, W, 3, device="cuda"), n, grad2d)
+    ctx.sync()
+    # colour gradients: the sum of the alphas taken in the tile, 256 terms of a few 1e-3
+    ref = torch.where(taken, alpha, torch.zeros_like(alpha)).double().reshape(H // 16, 16, W // 16, 16).sum((1, 3))
+    assert torch.allclose(grad2d[:, 6].double(), ref.reshape(-1), rtol=256 * 2.0 ** -24, atol=0.0)
+
+
+def test_render_takes_everything_without_a_least_alpha(ctx):
+    """alpha_min = 0 takes every entry of sigma >= 0, an opacity of 0 (whose opacity gradient is not 0)
+    and an infinite one (whose alpha is alpha_max everywhere) among them."""
+    W, H = 48, 16
+    co = torch.tensor([[0.1, 0.0, 0.1, 0.0], [0.1, 0.0, 0.1, 0.5], [30.0, 0.0, 30.0, float("inf")]])
+    uv = torch.tensor([[8.0, 8.0], [24.0, 8.0], [40.0, 8.0]])
+    proj, tiles = one_entry_per_tile(W, H, uv, co)
+    cam = ab.camera(sg.look_at((0.0, -5.0, 0.0), np.zeros(3), W, H))
+    out, st = torch.empty(H, W, 4, device="cuda"), ab.FwdState.alloc(W, H)
+    for alpha_min in (0.0, 1.0 / 255.0):
+        opts = ab.render_opts(alpha_min=alpha_min)
+        ab.abcd_render_composite_fwd(ctx, cam, opts, proj, tiles, None, None, ab.ABCD_F16, None, out, st)
+        grad2d = torch.empty(3, 9, device="cuda")
+        ab.abcd_render_backward(ctx, cam, opts, proj, tiles, None, None, ab.ABCD_F16, None, st,
+                                torch.ones(H, W, 3, device="cuda"), 3, grad2d)
+        ctx.sync()
+        last = st.n_last.reshape(H, 3, 16)
+        assert bool((last[:, 2] == 1).all()) and bool((st.A_T[:, 32:, 0] == np.float32(0.99)).all())
+        if alpha_min > 0:
+            assert bool((last[:, 0] == 0).all()) and bool((grad2d[0] == 0).all())
+        else:
+            ys, xs = np.mgrid[0:16, 0:16] + 0.5
+            e = np.exp(-0.05 * ((xs - 8.0) ** 2 + (ys - 8.0) ** 2))
+            assert bool((last[:, :2] == 1).all())
+            assert abs(float(grad2d[0, 5]) - 3.0 * e.sum()) <= 1e-5 * 3.0 * e.sum()
+            assert bool((grad2d[0, :5] == 0).all()) and bool((grad2d[0, 6:] == 0).all())
+
+
 @pytest.mark.parametrize("cam_idx", [0, 2])
 def test_render_backward_matches_oracle(ctx, tiny, cam_idx):
     case = Case(tiny, cam_idx, fb=True)
