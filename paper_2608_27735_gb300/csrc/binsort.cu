@@ -97,6 +97,8 @@ __device__ __forceinline__ void clear_rows(unsigned* rows_zero, int rows_words, 
 // the tile rectangles.  Up to kRankMax items, where the comparisons overtake the passes:
 // abcd_bin_sort 31 against 40 us with 1,000 Gaussians, 32 against 42 with 2,000, 37 against 49
 // with 4,000, 45 against 51 with 6,000; with 8,192 the counting took 18 us more than the passes.
+// CTAs are added where clearing the difference array takes more than the items do (4,096 cells each,
+// as keys_rects_kernel has them): 16 Gaussians at 16000x4000 463 -> 447 us, at 4096x2160 80 -> 78.
 constexpr int kRankMax = 6144;
 constexpr int kRankThreads = 256;
 
@@ -108,6 +110,7 @@ rank_sort_kernel(const float* depth, const int* radius, const float2* uv, int n,
   extern __shared__ __align__(16) unsigned s_key[];  // [n rounded up to 4], all ones past n
   clear_rows(rows_zero, rows_words, diff_zero, diff_cells, zero_word);
   const int first = blockIdx.x * per, quads = (n + 3) / 4;
+  if (first >= n) return;                            // launched for the clearing alone
   constexpr int kBatch = 8;                          // items a thread has in flight
   for (int b0 = 0; b0 < 4 * quads; b0 += kBatch * kRankThreads) {
     float2 m[kBatch];
@@ -1448,8 +1451,9 @@ abcd_status abcd::bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n, con
     const size_t smem = sizeof(uint4) * (size_t)((n + 3) / 4);
     by_depth = ctx->ws.dsort[0];
     if ((s = check_launch(ctx, "rank_sort_kernel",
-                          launch_pdl(rank_sort_kernel, dim3((n + per - 1) / per), dim3(kRankThreads),
-                                     smem, ctx->stream, (const float*)proj->depth,
+                          launch_pdl(rank_sort_kernel,
+                                     dim3((unsigned)std::max((n + per - 1) / per, (cells + 4095) / 4096)),
+                                     dim3(kRankThreads), smem, ctx->stream, (const float*)proj->depth,
                                      (const int*)proj->radius, (const float2*)proj->uv, n, per,
                                      tiles_x, tiles_y, by_depth, ctx->ws.rects, ctx->ws.row_runs,
                                      by_runs ? tiles_y : 0, ctx->ws.diff, cells, zero_word))))

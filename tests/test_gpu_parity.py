@@ -1281,6 +1281,43 @@ def test_small_blocks_order_as_the_radix_sort(ctx, n, depths):
     assert n < 64 or got[0][0] > 0
 
 
+@pytest.mark.parametrize("n", [1, 16, 17, 2000])
+@pytest.mark.parametrize("W,H", [(4200, 96), (16000, 4000)])
+def test_small_blocks_in_large_images(ctx, n, W, H):
+    """Few Gaussians on tile grids that take more CTAs to clear than to sort, the second one binned
+    without tile-row runs: three calls in turn, each with the cells the one before has left, give the
+    lists of the radix passes, and one CTA's worth of Gaussians take no longer than there (0.99 of the
+    time at 16000x4000; 1.025 with one CTA clearing 250,000 cells)."""
+    ctx.reserve(6200, 2_000_000, W * H)
+    cam = ab.camera(sg.look_at((0.0, -5.0, 0.0), np.zeros(3), W, H))
+    proj = ab.Projected.alloc(n)
+    proj.conic_opacity.copy_(torch.tensor([0.001, 0.0, 0.001, 0.9], device="cuda").expand(n, 4))
+    proj.radius.fill_(90)
+    tiles = ab.Tiles.alloc(1_000_000, W, H)
+    for k in range(3):
+        g = torch.Generator(device="cuda").manual_seed(10 * n + k)
+        proj.uv.copy_(torch.rand(n, 2, generator=g, device="cuda") * torch.tensor([W * 1.0, H * 1.0], device="cuda"))
+        proj.depth.copy_(0.2 + torch.rand(n, generator=g, device="cuda"))
+        got = []
+        for hook in (-1, 1 << 40):
+            assert ab.lib().abcd_test_withhold_lookback(ctx.h, hook) == ab.ABCD_OK
+            ab.abcd_bin_sort(ctx, proj, n, cam, tiles)
+            ctx.sync()
+            K = int(tiles.count.item())
+            got.append((K, tiles.ids[:K].clone(), tiles.ranges.clone()))
+        assert got[0][0] == got[1][0] > 0 and torch.equal(got[0][1], got[1][1]) and torch.equal(got[0][2], got[1][2])
+
+    if n > 16:
+        return
+
+    def hooked():
+        ab.lib().abcd_test_withhold_lookback(ctx.h, 1 << 40)
+        ab.abcd_bin_sort(ctx, proj, n, cam, tiles)
+
+    t = best_time(ctx, [lambda: ab.abcd_bin_sort(ctx, proj, n, cam, tiles), hooked])
+    assert t[0] <= 1.01 * t[1], t
+
+
 @pytest.mark.parametrize("over", [0, 1])
 def test_bin_sort_at_the_resident_limit(over):
     """The largest sort whose radix tiles and placement chunks are taken by CTA index, and one
