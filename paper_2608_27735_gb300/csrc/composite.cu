@@ -230,8 +230,8 @@ constexpr int kListCtas = 9;
 // round of loads of the tile's map entries, one of its layers.  Against the list at 1080p, 0.4 / 0.9
 // of the tiles stored: 1 and 1 layers 11.1 / 12.5 against 12.1 / 16.3 us, 4 and 4 15.0 / 22.1 against
 // 16.7 / 24.0.  With 5 and 5 a second round of both follows: 15.8 us against 11.8 (a tenth stored).
-// Four loads in flight and 12 CTAs per SM (40 registers): eight take 8.2 against 6.9 us for 3 layers,
-// 16 CTAs spill.
+// A fold of one layer into the accumulator, 0.9 stored: 13.2 against 15.6 us.  Four loads in flight
+// and 12 CTAs per SM (40 registers): eight take 8.2 against 6.9 us for 3 layers, 16 CTAs spill.
 constexpr int kShortLayers = 4;
 constexpr int kShortInFlight = 4;
 constexpr int kShortCtas = 12;
@@ -404,17 +404,20 @@ composite_packed_kernel(const __grid_constant__ PackedTable pt, int nf, int nb, 
 // One side's left fold continued from an fp32 accumulator: acc = acc over the listed layers, in
 // order (acc_in NULL: from transparent); the accumulator goes back in fp32 (acc_out) and/or as
 // its fp16 rounding (out16).  The fold runs the same fp32 operations in the same order as
-// composite_packed_kernel, so folding the layers in pieces gives its result bit for bit.
-__global__ void __launch_bounds__(kPackedThreads)
+// composite_packed_kernel, so folding the layers in pieces gives its result bit for bit; SHORT as there.
+template <bool SHORT>
+__global__ void __launch_bounds__(kPackedThreads, SHORT ? kShortCtas : kListCtas)
 fold_packed_kernel(const __grid_constant__ PackedTable pt, int n, int width, int height,
                    int tiles_x, const float4* acc_in, float4* acc_out, uint2* out16) {
   pdl_wait();
-  __shared__ int s_map[kMaxLayers], s_list[kMaxLayers], s_count;
+  __shared__ Stored s_list[SHORT ? 1 : kMaxLayers];
+  __shared__ int s_end;
   const int tile = blockIdx.x;
   const int unit = threadIdx.x;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) s_map[k] = __ldg(pt.map[k] + tile);
-  __syncthreads();
-  compact_stored(s_map, 0, n, unit, s_list, &s_count);
+  if (!SHORT && unit < 32) {
+    const int k = list_stored(pt, 0, n, tile, s_list);
+    if (unit == 0) s_end = k;
+  }
   const int r = unit / (kTile / 2), c = 2 * (unit % (kTile / 2));
   const int y = (tile / tiles_x) * kTile + r, x = (tile % tiles_x) * kTile + c;
   const long long p0 = (long long)y * width + x;
@@ -426,12 +429,12 @@ fold_packed_kernel(const __grid_constant__ PackedTable pt, int n, int width, int
     if (in0) { const float4 a = acc_in[p0]; acc[0] = a.x; acc[1] = a.y; acc[2] = a.z; acc[3] = a.w; }
     if (in1) { const float4 a = acc_in[p0 + 1]; acc[4] = a.x; acc[5] = a.y; acc[6] = a.z; acc[7] = a.w; }
   }
-  __syncthreads();
-  for_each_listed(pt.data, s_map, s_list, 0, s_count, unit, [&](int, uint4 v) {
-    float f[8];
-    unpack_h8(v, f);
-    fold<2>(acc, f);
-  });
+  if (SHORT) {
+    fold_short(pt, 0, n, tile, unit, acc);
+  } else {
+    __syncthreads();
+    fold_listed(pt, s_list, 0, s_end, unit, acc);
+  }
   if (in0) {
     if (acc_out) acc_out[p0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
     if (out16) store_pixel_out(out16, 1, p0, acc);
@@ -468,8 +471,9 @@ extern "C" abcd_status abcd_composite_fold_packed(abcd_ctx* ctx, const int* cons
   if (!acc_out && !out16) return ABCD_OK;
   const int tiles_x = (width + kTile - 1) / kTile, tiles_y = (height + kTile - 1) / kTile;
   return check_launch(ctx, "fold_packed_kernel",
-                      launch_pdl(fold_packed_kernel, dim3(tiles_x * tiles_y), dim3(kPackedThreads),
-                                 0, ctx->stream, pt, count, width, height, tiles_x,
+                      launch_pdl(count <= kShortLayers ? fold_packed_kernel<true> : fold_packed_kernel<false>,
+                                 dim3(tiles_x * tiles_y), dim3(kPackedThreads), 0, ctx->stream, pt, count,
+                                 width, height, tiles_x,
                                  (const float4*)acc_in, (float4*)acc_out, (uint2*)out16));
 }
 
