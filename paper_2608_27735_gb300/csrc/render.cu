@@ -654,7 +654,9 @@ __device__ __forceinline__ void load_pixel_grad(const BwdArgs& a, long long p, i
 // C the colour accumulated up to and including the entry.  The two pixels' arithmetic is paired
 // through the packed two-lane fp32 instructions, which have no negated operands: the staged
 // opacity is negated, and so is the replayed G . C, so that none is needed.  The decisions
-// (sigma, its limit) are rounded exactly as the forward rounds them.  Returns whether the entry
+// (sigma, its limit) are rounded exactly as the forward rounds them.  An entry that a pixel does not
+// take adds zeros by its weight of 0, which an infinite or NaN gradient of the pixel would turn into
+// NaN: blocks with such a pixel run with WILD, which selects the zeros.  Returns whether the entry
 // contributed to either pixel.
 constexpr int kSums = 6;              // sums per entry
 
@@ -662,7 +664,7 @@ struct PixB2 {
   float2 T, nGc, Gr, Gg, Gb, K;
 };
 
-template <bool CLAMP>
+template <bool CLAMP, bool WILD>
 __device__ __forceinline__ bool pixel_backward2(PixB2& p, const Entry& e, float2 sg, float2 dx,
                                                 bool live0, bool live1, const Opts& op,
                                                 float (&v)[kSums]) {
@@ -678,21 +680,29 @@ __device__ __forceinline__ bool pixel_backward2(PixB2& p, const Entry& e, float2
   const float2 gcol = __ffma2_rn(p.Gb, make_float2(e.col.z, e.col.z),
                                  __ffma2_rn(p.Gg, make_float2(e.col.y, e.col.y),
                                             __fmul2_rn(p.Gr, make_float2(e.col.x, e.col.x))));
-  p.nGc = __ffma2_rn(nw, gcol, p.nGc);                               // -G . C including the entry
+  const float2 nGc = __ffma2_rn(nw, gcol, p.nGc);                    // -G . C including the entry
+  p.nGc = WILD ? make_float2(ok0 ? nGc.x : p.nGc.x, ok1 ? nGc.y : p.nGc.y) : nGc;
   const float2 oma = __fadd2_rn(make_float2(1.f, 1.f), na);
   const float2 nioma = make_float2(rcp_approx(-oma.x), rcp_approx(-oma.y));
   const float2 km = __fadd2_rn(p.K, p.nGc);
   float2 da = __ffma2_rn(km, nioma, __fmul2_rn(p.T, gcol));
   // d alpha / d opacity = G, d alpha / d sigma = -alpha; none of either where alpha was clamped
   if (CLAMP) da = make_float2(nraw.x >= -op.alpha_max ? da.x : 0.f, nraw.y >= -op.alpha_max ? da.y : 0.f);
+  if (WILD) da = make_float2(ok0 ? da.x : 0.f, ok1 ? da.y : 0.f);
   const float2 dg = __fmul2_rn(da, G);
   const float2 t = __fmul2_rn(__fmul2_rn(da, nraw), dx);             // dL/dsigma dx
   v[0] = dg.x + dg.y;
   v[1] = t.x + t.y;
   v[2] = fmaf(t.x, dx.x, t.y * dx.y);
-  v[3] = fmaf(p.Gr.x, -nw.x, p.Gr.y * -nw.y);
-  v[4] = fmaf(p.Gg.x, -nw.x, p.Gg.y * -nw.y);
-  v[5] = fmaf(p.Gb.x, -nw.x, p.Gb.y * -nw.y);
+  if (WILD) {
+    v[3] = (ok0 ? p.Gr.x * -nw.x : 0.f) + (ok1 ? p.Gr.y * -nw.y : 0.f);
+    v[4] = (ok0 ? p.Gg.x * -nw.x : 0.f) + (ok1 ? p.Gg.y * -nw.y : 0.f);
+    v[5] = (ok0 ? p.Gb.x * -nw.x : 0.f) + (ok1 ? p.Gb.y * -nw.y : 0.f);
+  } else {
+    v[3] = fmaf(p.Gr.x, -nw.x, p.Gr.y * -nw.y);
+    v[4] = fmaf(p.Gg.x, -nw.x, p.Gg.y * -nw.y);
+    v[5] = fmaf(p.Gb.x, -nw.x, p.Gb.y * -nw.y);
+  }
   p.T = __fmul2_rn(p.T, oma);
   return ok0 || ok1;
 }
@@ -708,7 +718,7 @@ __device__ __forceinline__ bool pixel_backward2(PixB2& p, const Entry& e, float2
 constexpr int kRedPitch = 36;
 static_assert(kBwdUnroll * kSums <= 32, "one row per lane");
 
-template <bool CLAMP>
+template <bool CLAMP, bool WILD>
 __device__ __forceinline__ void bwd_staged(const BwdArgs& a, PixB2& pp, float2 fx, float fy,
                                            float by0, unsigned last0, unsigned last1, int cnt,
                                            const float4* s_co, const float4* s_m,
@@ -725,7 +735,7 @@ __device__ __forceinline__ void bwd_staged(const BwdArgs& a, PixB2& pp, float2 f
       float2 dx, sg;
       float dy, v[kSums];
       sigma_pair(e.s, e.m, fx, fy, dx, dy, sg);
-      const bool c = pixel_backward2<CLAMP>(pp, e, sg, dx, nxt <= last0, nxt <= last1, a.op, v);
+      const bool c = pixel_backward2<CLAMP, WILD>(pp, e, sg, dx, nxt <= last0, nxt <= last1, a.op, v);
       if (__any_sync(0xffffffffu, c)) who |= 1u << i;
 #pragma unroll
       for (int k = 0; k < kSums; ++k) s_red[(kSums * i + k) * kRedPitch + lane] = v[k];
@@ -794,14 +804,18 @@ __device__ __forceinline__ void bwd_chunk(const BwdArgs& a, int blk, int start, 
   pp.Gb = make_float2(p0.Gb, p1.Gb);
   pp.K = make_float2(p0.K, p1.K);
   const unsigned last0 = p0.last, last1 = p1.last;
+  const float size0 = fabsf(p0.Gr) + fabsf(p0.Gg) + fabsf(p0.Gb) + fabsf(p0.K);
+  const float size1 = fabsf(p1.Gr) + fabsf(p1.Gg) + fabsf(p1.Gb) + fabsf(p1.K);
+  const bool wild = __any_sync(0xffffffffu, !(size0 + size1 < 3.402823466e38f));
   int next = start;
   while (next < span) {
     __syncwarp();
     bool clamp;
     const int cnt = stage_fill(a.ids, rg.x, span, next, a.uv, a.co, a.rgb, bx0, by0, a.op, s_co,
                                s_m, s_rgb, s_id, clamp);
-    if (!clamp) bwd_staged<false>(a, pp, fx, fy, by0, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
-    else bwd_staged<true>(a, pp, fx, fy, by0, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
+    if (wild) bwd_staged<true, true>(a, pp, fx, fy, by0, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
+    else if (clamp) bwd_staged<true, false>(a, pp, fx, fy, by0, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
+    else bwd_staged<false, false>(a, pp, fx, fy, by0, last0, last1, cnt, s_co, s_m, s_rgb, s_id, s_red);
   }
 }
 

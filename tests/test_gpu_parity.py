@@ -444,6 +444,38 @@ def test_render_limit_decides_as_the_alpha(ctx, lo, hi):
     assert torch.allclose(grad2d[:, 6].double(), ref.reshape(-1), rtol=256 * 2.0 ** -24, atol=0.0)
 
 
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+def test_render_backward_keeps_a_bad_pixel_to_its_entries(ctx, bad):
+    """A gradient that is not finite at one pixel reaches the entries that the pixel takes, and no other
+    entry of its 8x8 block."""
+    W, H = 16, 16
+    uv = torch.tensor([[2.5, 2.5], [5.5, 5.5], [12.5, 4.5]])
+    co = torch.tensor([[2.0, 0.0, 2.0, 0.9], [2.0, 0.3, 2.0, 0.8], [0.05, 0.0, 0.05, 0.999]])
+    proj = ab.Projected.alloc(3)
+    proj.uv.copy_(uv)
+    proj.conic_opacity.copy_(co)
+    proj.rgb.copy_(torch.tensor([[1.0, 0.5, 0.2], [0.3, 0.9, 0.4], [0.2, 0.1, 0.6]]))
+    tiles = ab.Tiles.alloc(8, W, H)
+    tiles.ids[:3] = torch.tensor([0, 1, 2], dtype=torch.int32)
+    tiles.ranges.copy_(torch.tensor([[0, 3]], dtype=torch.int32))
+    cam = ab.camera(sg.look_at((0.0, -5.0, 0.0), np.zeros(3), W, H))
+    out, st = torch.empty(H, W, 4, device="cuda"), ab.FwdState.alloc(W, H)
+    ab.abcd_render_composite_fwd(ctx, cam, None, proj, tiles, None, None, ab.ABCD_F16, None, out, st)
+    got = []
+    for v in (0.0, bad):
+        dl = torch.rand(H, W, 3, generator=torch.Generator().manual_seed(1)).cuda()
+        dl[0, 0] = v                                   # only entry 2's tail reaches this corner
+        dl[2, 2, 1] = v
+        grad2d = torch.empty(3, 9, device="cuda")
+        ab.abcd_render_backward(ctx, cam, None, proj, tiles, None, None, ab.ABCD_F16, None, st, dl, 3, grad2d)
+        ctx.sync()
+        got.append(grad2d)
+    assert bool(torch.isfinite(got[0]).all()) and bool((got[0][1] != 0).any())
+    assert bool(torch.isfinite(got[1][1]).all())
+    assert torch.allclose(got[1][1], got[0][1], rtol=1e-5, atol=1e-7)
+    assert not bool(torch.isfinite(got[1][0]).all()) and not bool(torch.isfinite(got[1][2]).all())
+
+
 def test_render_takes_everything_without_a_least_alpha(ctx):
     """alpha_min = 0 takes every entry of sigma >= 0, an opacity of 0 (whose opacity gradient is not 0)
     and an infinite one (whose alpha is alpha_max everywhere) among them."""
