@@ -22,6 +22,9 @@ constexpr long long kMaxDiffCells = 1LL << 20;   // (tiles_x + 1) * (tiles_y + 1
 constexpr int kMaxRunRows = 1024;     // tile grids that bin through tile-row runs: rows ...
 constexpr int kMaxRunCols = 256;      // ... and columns at most
 constexpr int kVisSumCopies = 8;          // copies of the layer visibility sums
+// words of Workspace::os_ctr: [2 sorts][2] tile and finished-CTA counters of a radix pass, the run
+// placement's two, [2 calls in turn][2] the visible depth keys' range, the count kernel's finished CTAs
+constexpr int kCtrSorts = 0, kCtrPlace = 4, kCtrKeyRange = 8, kCtrTicket = 12;
 constexpr int kSmemKernels = 16;          // kernels with dynamic shared memory, at most
 
 // Device status bits (OR-ed into the status word; abcd_sync reports the lowest set code).
@@ -50,7 +53,7 @@ struct Workspace {
   unsigned long long* dsort[2];     // depth sort items [max_g]
   unsigned long long* pairs[2];     // (tile << 32 | id) items [max_pairs]
   unsigned* os_gh;                  // [2 sorts][4 passes][kRadixBins] digit counts
-  unsigned* os_ctr;                 // [2 sorts][2] tile and finished-CTA counters of a pass
+  unsigned* os_ctr;                 // the binning's counters (kCtr...), zero or ready between calls
   unsigned long long* os_state;     // [os_tiles][kRadixBins] look-back words
   long long os_tiles;
   int4* rects;                      // [max_g] tile rectangle per Gaussian

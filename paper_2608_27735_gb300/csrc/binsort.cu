@@ -14,10 +14,12 @@
 //      tiles in each of its tile rows (the kept set is convex), its pair (or run) count, and
 //      +-1 at the run's ends in a per-row difference array over the tile grid (block-local
 //      first);
-//   2. stable LSD radix sort of the n Gaussians by the 32 depth bits, on the context's side
-//      stream, while the main stream makes the row runs and then, in one block, the tile
-//      ranges (row prefix sums of the difference array, an exclusive scan, K) and the tiles
-//      ordered by decreasing pair count (the order the render kernels launch them in);
+//   2. stable LSD radix sort of the n Gaussians by the 32 depth bits, on the context's stream,
+//      while its side stream makes the row runs and then, in one block, the tile ranges (row
+//      prefix sums of the difference array, an exclusive scan, K) and the tiles ordered by
+//      decreasing pair count (the order the render kernels launch them in); up to 6,144 Gaussians
+//      are ordered by counting instead, in the kernel of step 1's rectangles, and everything
+//      follows on the one stream;
 //   3. exclusive scan of the pair (run) counts in depth order: every Gaussian's output offset;
 //   4. for tile grids up to 256 x 1024 tiles: emission of one item per non-empty (Gaussian,
 //      tile row) run in depth order (row, x0, x1, id; the runs are recomputed with the same
@@ -32,8 +34,8 @@
 //      of equal width, which keeps depth order inside each tile; the last pass writes ids.
 // Radix sorts are one-sweep: one kernel counts the digits of all passes, then each pass is a
 // single kernel whose CTAs take tiles of items in order and find the offsets of their digits
-// by decoupled look-back over the tiles before theirs (bounded waits on CTAs that are already
-// running).  Lanes of equal digit are ranked with ballots on the low, scattered digits and
+// by decoupled look-back over the tiles before theirs (bounded waits on CTAs that have claimed
+// their tiles or, where all fit at once, have lower indices).  Lanes of equal digit are ranked with ballots on the low, scattered digits and
 // with __match_any_sync on the high, grouped ones.
 // Counts that live on the device (K) are read by the kernels themselves; grids are fixed, so
 // the step has no host sync.
@@ -445,14 +447,15 @@ __device__ __forceinline__ unsigned rank_peers(unsigned d, bool valid) {
 
 // ---- one-sweep radix sort (decoupled look-back)
 // A sort of n items on bits [bit_lo, bit_hi) runs in passes of equal width.  One kernel counts
-// the digits of every pass at once; then each pass is a single kernel: CTAs claim tiles of
-// kOsWarps x 32 x U consecutive items in order (a global counter), rank each item among the
-// tile's items of equal digit (stable), publish the tile's per-digit counts, and add up the
+// the digits of every pass at once; then each pass is a single kernel: CTAs take tiles of
+// kOsWarps x 32 x U consecutive items in order (from a global counter, or each its own when they
+// are all resident at once), rank each item among the tile's items of equal digit (stable), publish the tile's per-digit counts, and add up the
 // counts of the tiles before theirs by looking back until a tile whose inclusive prefix is
 // published.  Item position = digit base + prefix of earlier tiles + rank in the tile.
-// A tile only waits for tiles claimed before it, whose CTAs are running, so the waits end;
-// each is bounded all the same (on expiry the status word gets ABCD_ERR_TIMEOUT and the pass
-// goes on with a wrong prefix instead of hanging).
+// A claimed tile only waits for tiles claimed before it, whose CTAs are running, so the waits end.
+// A CTA that takes the tile of its own index waits for CTAs of lower indices, and that those have
+// started is how GPUs hand out CTAs, not what CUDA promises.  Each wait is therefore bounded: on expiry
+// the status word gets ABCD_ERR_TIMEOUT and the pass goes on with a wrong prefix instead of hanging.
 struct SortPasses {
   int n;                 // passes (at most kMaxSortPasses)
   int shift[4];          // low bit of each pass's digit
@@ -573,8 +576,8 @@ onesweep_kernel(const T* in, T* out, unsigned* out_ids, unsigned id_mask, long l
   const unsigned lt = (1u << lane) - 1u;
   const KeyMap km = key_map(krange);
   // Tiles that are all resident at once need no claims: CTA b takes tile b.  The tiles it waits
-  // for have lower CTA indices and were started before it; the wait's bound also covers a start
-  // in another order with the SMs full of other streams' work.  That saves three round trips per
+  // for have lower CTA indices, which start first (see above; the wait's bound covers a start in
+  // another order with the SMs full of other streams' work).  That saves three round trips per
   // pass (the claim, the claim that finds nothing left, the counters' reset): a pass over 100,000
   // keys 12.0 -> 10.2 us, abcd_bin_sort 93 -> 82 us there.
   const bool fixed = n_tiles <= (long long)resident;
@@ -1126,7 +1129,8 @@ constexpr int kPlaceLB = 8;                          // look-back words read per
 static_assert(kMaxRunRows % kPlaceThreads == 0 && kPlaceRuns % kPlaceThreads == 0, "tiling");
 
 // Runs sorted by row (depth order inside a row) -> ids in the tile ranges.  row_runs: runs per
-// row; chunks are claimed in order through ctr (the last CTA clears it); state: tiles_x look-back
+// row; chunks are claimed in order through ctr (the last CTA clears it), or taken by CTA index when
+// they are all resident at once (as the radix passes' tiles); state: tiles_x look-back
 // words per chunk.  Inside a chunk, column x keeps a bit mask of the runs that cover it and the
 // number of covering runs before each mask word, so the rank of run j in column x is a
 // popcount.  A wait gives up after spin_limit polls (status gets ABCD_ERR_TIMEOUT).
@@ -1344,7 +1348,7 @@ abcd_status radix_sort(abcd_ctx* ctx, cudaStream_t st, T* a, T* b, long long n_s
   const SortPasses sp = make_passes(bit_lo, bit_hi);
   if (sp.n < 1 || sp.n > 4) return fail(ctx, ABCD_ERR_INVALID_ARG, "radix sort of %d bits", bit_hi - bit_lo);
   unsigned* gh = ctx->ws.os_gh + (size_t)slot * 4 * kRadixBins;
-  unsigned* ctr = ctx->ws.os_ctr + 2 * slot;
+  unsigned* ctr = ctx->ws.os_ctr + kCtrSorts + 2 * slot;
   const long long tile = (long long)kOsThreads * (64 / (int)sizeof(T));
   const long long tiles = (n_max + tile - 1) / tile;
   if (tiles > ctx->ws.os_tiles) return fail(ctx, ABCD_ERR_WORKSPACE, "radix sort: %lld tiles exceed the workspace", tiles);
@@ -1421,8 +1425,8 @@ abcd_status abcd::bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n, con
   abcd_status s;
   // the visible depth keys' range: two pairs of words used in turn, each call's keys_rects
   // clearing the other pair for the next call (zero initially: the workspace set-up clears them)
-  unsigned* krange = ctx->ws.os_ctr + 8 + 2 * (int)(ctx->krange_parity & 1u);
-  unsigned* krange_next = ctx->ws.os_ctr + 8 + 2 * (int)((ctx->krange_parity + 1u) & 1u);
+  unsigned* krange = ctx->ws.os_ctr + kCtrKeyRange + 2 * (int)(ctx->krange_parity & 1u);
+  unsigned* krange_next = ctx->ws.os_ctr + kCtrKeyRange + 2 * (int)((ctx->krange_parity + 1u) & 1u);
   const float alpha_min = make_opts(opts).alpha_min;
   int tile_bits = 1;
   while ((1LL << tile_bits) < n_tiles) ++tile_bits;
@@ -1536,7 +1540,7 @@ abcd_status abcd::bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n, con
                                    (const u64*)by_depth, n, (const unsigned*)ctx->ws.counts,
                                    ctx->ws.block_sums, Ge,
                                    by_runs ? ctx->ws.n_runs : (long long*)out->count, cap,
-                                   ctx->ws.status, ctx->ws.os_ctr + 12))))
+                                   ctx->ws.status, ctx->ws.os_ctr + kCtrTicket))))
     return s;
   if (by_runs) {
     u64* runs = ctx->ws.pairs[0];
@@ -1568,7 +1572,7 @@ abcd_status abcd::bin_sort(abcd_ctx* ctx, const abcd_projected* proj, int n, con
                                    (const u64*)by_row, (const long long*)ctx->ws.n_runs, cap,
                                    (const unsigned*)ctx->ws.row_runs, tiles_y, tiles_x,
                                    (const unsigned*)out->ranges, (const long long*)out->count,
-                                   (unsigned*)out->ids, ctx->ws.os_state, ctx->ws.os_ctr + 4, epoch,
+                                   (unsigned*)out->ids, ctx->ws.os_state, ctx->ws.os_ctr + kCtrPlace, epoch,
                                    ctx->ws.status, ctx->wait_limit, resident));
   }
   int id_bits = 1;

@@ -308,8 +308,8 @@ struct PixF2 {
 
 // One staged list entry as the backward's loop reads it.
 struct Entry {
-  float4 s;            // scaled conic, opacity
-  float4 m;            // uv, sigma limit, list position + 1 (bits)
+  float4 s;            // scaled conic, opacity negated
+  float4 m;            // uv negated, sigma limit, list position + 1 (bits)
   float4 col;          // rgb
 };
 
